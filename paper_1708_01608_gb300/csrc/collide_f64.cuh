@@ -1,0 +1,169 @@
+// The FP64 collision of one cell, counted in FP64 instructions.
+//
+// GB300 issues two FP64 lanes per SM and cycle (1.25 TFLOP/s over 152 SMs),
+// so an FP64 step is bound by that pipe long before HBM: at 128^3 the 304
+// bytes of an update take 94 us per step at the copy bandwidth, the 549 FP64
+// instructions of the former velocity-by-velocity form took 2.285 ms.  This
+// form spends 169 (90 DADD, 14 DMUL, 65 DFMA, halo included): 0.734 ms, the
+// pipe 81 % busy (ncu); D2Q9 at 1024^2 went from 0.599 to 0.183 ms.  With w the edge weight (1/36),
+// m = rho u and one value each per axis a
+//   B_a = 3 omega w m_a,  v_a = 1.5 u_a,  Q_a = B_a v_a,
+//   K = omega w rho - (Q_x + Q_y + Q_z)/3,
+// omega f_eq of the rest, an axis and an edge velocity is
+//   R0 K,  R (K + Q_a) +- R B_a,
+//   K + Q_a + Q_b + c_a c_b B_a (2 v_b) +- (c_a B_a + c_b B_b)
+// (R and R0 the weights' ratios 2 and 12, D2Q9 4 and 16), so opposite
+// velocities share the even part, the four edges of a plane share
+// K + Q_a + Q_b, relaxation is one FMA on (1 - omega) f_i, and the only
+// division left is one reciprocal of rho.  Zero velocity components cost
+// nothing (a product with 0.0 is not removable under IEEE rules) and the
+// density is the psi phase's sum.
+#pragma once
+
+#include "lattice.cuh"
+
+namespace sclbm {
+
+// 2^(k/64), k = 0 .. 63, rounded to nearest
+static __device__ const double EXP2_64TH[64] = {
+    0x1.0000000000000p+0, 0x1.02c9a3e778061p+0, 0x1.059b0d3158574p+0, 0x1.0874518759bc8p+0,
+    0x1.0b5586cf9890fp+0, 0x1.0e3ec32d3d1a2p+0, 0x1.11301d0125b51p+0, 0x1.1429aaea92de0p+0,
+    0x1.172b83c7d517bp+0, 0x1.1a35beb6fcb75p+0, 0x1.1d4873168b9aap+0, 0x1.2063b88628cd6p+0,
+    0x1.2387a6e756238p+0, 0x1.26b4565e27cddp+0, 0x1.29e9df51fdee1p+0, 0x1.2d285a6e4030bp+0,
+    0x1.306fe0a31b715p+0, 0x1.33c08b26416ffp+0, 0x1.371a7373aa9cbp+0, 0x1.3a7db34e59ff7p+0,
+    0x1.3dea64c123422p+0, 0x1.4160a21f72e2ap+0, 0x1.44e086061892dp+0, 0x1.486a2b5c13cd0p+0,
+    0x1.4bfdad5362a27p+0, 0x1.4f9b2769d2ca7p+0, 0x1.5342b569d4f82p+0, 0x1.56f4736b527dap+0,
+    0x1.5ab07dd485429p+0, 0x1.5e76f15ad2148p+0, 0x1.6247eb03a5585p+0, 0x1.6623882552225p+0,
+    0x1.6a09e667f3bcdp+0, 0x1.6dfb23c651a2fp+0, 0x1.71f75e8ec5f74p+0, 0x1.75feb564267c9p+0,
+    0x1.7a11473eb0187p+0, 0x1.7e2f336cf4e62p+0, 0x1.82589994cce13p+0, 0x1.868d99b4492edp+0,
+    0x1.8ace5422aa0dbp+0, 0x1.8f1ae99157736p+0, 0x1.93737b0cdc5e5p+0, 0x1.97d829fde4e50p+0,
+    0x1.9c49182a3f090p+0, 0x1.a0c667b5de565p+0, 0x1.a5503b23e255dp+0, 0x1.a9e6b5579fdbfp+0,
+    0x1.ae89f995ad3adp+0, 0x1.b33a2b84f15fbp+0, 0x1.b7f76f2fb5e47p+0, 0x1.bcc1e904bc1d2p+0,
+    0x1.c199bdd85529cp+0, 0x1.c67f12e57d14bp+0, 0x1.cb720dcef9069p+0, 0x1.d072d4a07897cp+0,
+    0x1.d5818dcfba487p+0, 0x1.da9e603db3285p+0, 0x1.dfc97337b9b5fp+0, 0x1.e502ee78b3ff6p+0,
+    0x1.ea4afa2a490dap+0, 0x1.efa1bee615a27p+0, 0x1.f50765b6e4540p+0, 0x1.fa7c1819e90d8p+0};
+
+// psi(rho) = rho0 (1 - exp(-rho/rho0)) with the table-driven exponential of
+// Tang (ACM TOMS 15, 1989): x = n ln2/64 + r with |r| <= ln2/128, e^x =
+// 2^(n/64) (1 + r + r^2/2 + ... + r^5/120), the tail below 4e-17.  12 FP64
+// instructions against about 20 with exp() (128^3: 0.786 to 0.743 ms, the
+// density in two chains included).  The range test is on integers;
+// outside it (and for NaN) exp() decides.
+__device__ __forceinline__ double psi_f64(double rho, double rho0, double inv_rho0) {
+  const double x = -rho * inv_rho0;
+  if ((__double2hiint(x) & 0x7fffffff) >= 0x4085e000) return rho0 * (1.0 - exp(x));  // |x| >= 700
+  const double t = fma(x, 0x1.71547652b82fep+6, 0x1.8p52);  // n in the low word
+  const int n = __double2loint(t);
+  const double nd = t - 0x1.8p52;
+  const double T = __ldg(EXP2_64TH + (n & 63));
+  const double r = fma(nd, -0x1.473de6af278edp-40, fma(nd, -0x1.62e42fefp-7, x));
+  double q = fma(r, 1.0 / 120.0, 1.0 / 24.0);
+  q = fma(q, r, 1.0 / 6.0);
+  q = fma(q, r, 0.5);
+  q = fma(q * r, r, r);  // e^r - 1
+  const double S = __hiloint2double(__double2hiint(T) + ((n >> 6) << 20), __double2loint(T));
+  return fma(-rho0, fma(S, q, S), rho0);
+}
+
+// Density of one cell from its Q values, in two chains (half the latency of
+// one; the owner and a neighbour's halo thread use the same order)
+template <int Q, class Ld>
+__device__ __forceinline__ double rho_f64(Ld ld) {
+  double a = ld(0), b = ld(1);
+#pragma unroll
+  for (int i = 2; i + 1 < Q; i += 2) {
+    a += ld(i);
+    b += ld(i + 1);
+  }
+  if constexpr (Q % 2 == 1) a += ld(Q - 1);
+  return a + b;
+}
+
+template <int LAT>
+struct RelaxF64 {
+  static constexpr double R = LAT == D3Q19 ? 2.0 : 4.0;     // axis weight / edge weight
+  static constexpr double R0 = LAT == D3Q19 ? 12.0 : 16.0;  // rest weight / edge weight
+  double om1, fG, wK, cB;
+  __device__ __forceinline__ RelaxF64(double tau, double G) {
+    const double omega = 1.0 / tau, w = 1.0 / 36.0;
+    om1 = 1.0 - omega;
+    fG = -tau * G * w;
+    wK = omega * w;
+    cB = 3.0 * omega * w;
+  }
+};
+
+template <int CC>
+__device__ __forceinline__ double cacc_d(double acc, double v) {
+  if constexpr (CC > 0) return acc + v;
+  else if constexpr (CC < 0) return acc - v;
+  else return acc;
+}
+
+// f(i): the cell's populations, rho their sum, psi0 and psi(i) the
+// pseudopotential here and at x + c_i; put(i, v) takes the collided
+// population (integral_constant i).  SITE adds w_i dm to every population.
+template <int LAT, bool SITE, class F, class Psi, class Put>
+__device__ __forceinline__ void collide_f64(const RelaxF64<LAT> &q, F f, double rho, double psi0,
+                                            Psi psi, Put put, double dm) {
+  using L = Lattice<LAT>;
+  constexpr double R = RelaxF64<LAT>::R, R0 = RelaxF64<LAT>::R0;
+  // -0 is the additive identity, so a first term is no addition
+  double j[3] = {-0.0, -0.0, -0.0}, ax[3] = {0.0, 0.0, 0.0}, ed[3] = {-0.0, -0.0, -0.0};
+  static_for<L::NP>([&](auto kc) {
+    constexpr int i = L::rep(decltype(kc)::value), o = L::opp(i);
+    constexpr int cx = L::cx(i), cy = L::cy(i), cz = L::cz(i);
+    constexpr bool axis = cx * cx + cy * cy + cz * cz == 1;
+    const double d = f(i) - f(o), dp = psi(i) - psi(o);
+    j[0] = cacc_d<cx>(j[0], d);
+    j[1] = cacc_d<cy>(j[1], d);
+    j[2] = cacc_d<cz>(j[2], d);
+    if constexpr (axis) {
+      static_assert(cx + cy + cz == 1, "axis representatives point along +a");
+      ax[cx ? 0 : (cy ? 1 : 2)] = dp;
+    } else {
+      ed[0] = cacc_d<cx>(ed[0], dp);
+      ed[1] = cacc_d<cy>(ed[1], dp);
+      ed[2] = cacc_d<cz>(ed[2], dp);
+    }
+  });
+  const double gp = q.fG * psi0, ir = 1.5 * __drcp_rn(rho);
+  double v[3], B[3], Q[3], s = -0.0;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    if (a == 1 && !L::HAS_Y) continue;
+    const double m = fma(gp, fma(R, ax[a], ed[a]), j[a]);
+    v[a] = m * ir;
+    B[a] = q.cB * m;
+    Q[a] = B[a] * v[a];
+    s += Q[a];
+  }
+  const double K = fma(s, -1.0 / 3.0, q.wK * rho);
+  auto out = [&](auto ic, double x) {
+    constexpr int i = decltype(ic)::value;
+    put(ic, SITE ? x + L::w(i) * dm : x);
+  };
+  out(std::integral_constant<int, 0>{}, fma(q.om1, f(0), R0 * K));
+  static_for<L::NP>([&](auto kc) {
+    constexpr int i = L::rep(decltype(kc)::value), o = L::opp(i);
+    constexpr int cx = L::cx(i), cy = L::cy(i), cz = L::cz(i);
+    constexpr int c[3] = {cx, cy, cz};
+    constexpr int a = cx ? 0 : (cy ? 1 : 2);
+    if constexpr (cx * cx + cy * cy + cz * cz == 1) {
+      const double A = R * (K + Q[a]);
+      out(std::integral_constant<int, i>{}, fma(R, B[a], fma(q.om1, f(i), A)));
+      out(std::integral_constant<int, o>{}, fma(-R, B[a], fma(q.om1, f(o), A)));
+    } else {
+      constexpr int b = cz ? 2 : 1;
+      const double D = (K + Q[a]) + Q[b], v2 = v[b] + v[b];
+      const double A = c[a] * c[b] > 0 ? fma(B[a], v2, D) : fma(-B[a], v2, D);
+      // c_a B_a + c_b B_b up to the sign of c_a
+      const double t = c[a] * c[b] > 0 ? B[a] + B[b] : B[a] - B[b];
+      const double hi = fma(q.om1, f(i), A), ho = fma(q.om1, f(o), A);
+      out(std::integral_constant<int, i>{}, c[a] > 0 ? hi + t : hi - t);
+      out(std::integral_constant<int, o>{}, c[a] > 0 ? ho - t : ho + t);
+    }
+  });
+}
+
+}  // namespace sclbm

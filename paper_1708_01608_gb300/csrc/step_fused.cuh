@@ -27,6 +27,7 @@
 #include <climits>
 #include <type_traits>
 
+#include "collide_f64.cuh"
 #include "internal.h"
 #include "lattice.cuh"
 
@@ -145,6 +146,13 @@ __device__ __forceinline__ bool fused_march(const MarchArgs &m, OutPop out_pop, 
   using C = typename K::C;
   constexpr int Q = K::Q, HY = K::HY, HX = K::HX, PW = K::PW, PH = K::PH, NT = K::NT;
   constexpr bool F64 = sizeof(C) == 8;
+  // FP64 holds one plane in registers: plane P is summed for psi straight
+  // from its stage and read into registers after the collision of P - 1, so
+  // its stage is free one iteration later and NS - 1 planes are in flight
+  // (a second register plane, 38 registers, spilled; the step is bound by
+  // the FP64 pipe and leaves the copies ample time).  FP32 arithmetic reads
+  // a plane once and has NS in flight.
+  constexpr bool KEEP = !F64;
   // 16-bit residual forms: the cell's rounding residual of the last step
   // joins its mass R, and the new one is what this step's stores round off
   constexpr bool RESID = S::RESID;
@@ -285,12 +293,12 @@ __device__ __forceinline__ bool fused_march(const MarchArgs &m, OutPop out_pop, 
   // The staged values of this thread's cell: FP64 keeps them per velocity;
   // the FP32 path keeps the opposite pairs (i, opp(i)) as float2 so that
   // their sums and relaxations run as paired FP32 instructions.
-  C cur[Q], nxt[Q];
+  C cur[F64 ? Q : 1];
   float2 cur2[L::NP], nxt2[L::NP];
   float cur0 = 0.0f, nxt0 = 0.0f;
   if constexpr (F64) {
 #pragma unroll
-    for (int i = 0; i < Q; ++i) cur[i] = nxt[i] = 0;
+    for (int i = 0; i < Q; ++i) cur[i] = 0;
   } else {
 #pragma unroll
     for (int k2 = 0; k2 < L::NP; ++k2) cur2[k2] = nxt2[k2] = make_float2(0.0f, 0.0f);
@@ -306,6 +314,8 @@ __device__ __forceinline__ bool fused_march(const MarchArgs &m, OutPop out_pop, 
     c3[k2] = (C)3 * w * omega;
     c45[k2] = (C)4.5 * w * omega;
   }
+
+  [[maybe_unused]] const RelaxF64<LAT> relax(m.tau, m.G);
 
   // two planes per iteration where registers allow (512-thread tiles): the
   // staged values then change register sets instead of being copied
@@ -323,12 +333,7 @@ __device__ __forceinline__ bool fused_march(const MarchArgs &m, OutPop out_pop, 
     if (active) {
       C rho = 0;
       if constexpr (F64) {
-#pragma unroll
-        for (int i = 0; i < Q; ++i) {
-          const C v = S::load(mainb[(i * BY + ty) * BX + tx]);
-          nxt[i] = v;
-          rho += v;
-        }
+        rho = rho_f64<Q>([&](int i) { return mainb[(i * BY + ty) * BX + tx]; });
       } else {
         static_for<L::NP>([&](auto kc) {
           constexpr int k2 = decltype(kc)::value, i = L::rep(k2), o = L::opp(i);
@@ -338,31 +343,42 @@ __device__ __forceinline__ bool fused_march(const MarchArgs &m, OutPop out_pop, 
         nxt0 = S::load(mainb[ty * BX + tx]);
         rho = rho_chain<Q>([&](int i) { return S::load(mainb[(i * BY + ty) * BX + tx]); });
       }
-      rk[(ty + HY) * PW + tx + 1] = psi_of(rho_ref + rho, rho0, inv_rho0);
+      if constexpr (F64)
+        rk[(ty + HY) * PW + tx + 1] = psi_f64(rho, rho0, inv_rho0);
+      else
+        rk[(ty + HY) * PW + tx + 1] = psi_of(rho_ref + rho, rho0, inv_rho0);
       Rnxt = rho;
     }
     if (tid < nhalo) {
       const T *b = reinterpret_cast<const T *>(st + h_off);
       C rho = 0;
       if constexpr (F64) {
-#pragma unroll
-        for (int i = 0; i < Q; ++i) rho += S::load(b[i * h_pstride]);
+        rho = rho_f64<Q>([&](int i) { return b[i * h_pstride]; });
       } else {
         rho = rho_chain<Q>([&](int i) { return S::load(b[i * h_pstride]); });
       }
-      rk[h_slot] = psi_of(rho_ref + rho, rho0, inv_rho0);
+      if constexpr (F64)
+        rk[h_slot] = psi_f64(rho, rho0, inv_rho0);
+      else
+        rk[h_slot] = psi_of(rho_ref + rho, rho0, inv_rho0);
     }
 
     if (__syncthreads_or(!ok)) {
       if (tid == 0) {
         if (m.err) atomicOr(m.err, ERR_TMA_TIMEOUT);
         // wait (bounded) for copies still in flight into this CTA's stages
-        for (int k2 = k + 1; k2 < NPL && k2 < k + NS; ++k2)
+        const int hi = KEEP ? min(NPL, k + NS) : min(NPL, max(NS, k + NS - 1));
+        for (int k2 = k + 1; k2 < hi; ++k2)
           mbar_wait_bounded(&bars[(k0 + k2) % NS], ((k0 + k2) / NS) & 1u, 100000000ull);
       }
       return false;
     }
-    if (tid == 0 && k + NS < NPL) issue(k + NS);
+    if constexpr (KEEP) {
+      if (tid == 0 && k + NS < NPL) issue(k + NS);
+    } else {
+      // the stage of plane P - 1 was last read before this barrier
+      if (tid == 0 && k >= 1 && k - 1 + NS < NPL) issue(k - 1 + NS);
+    }
 
     // ---- collide plane P - 1 (needs psi of P - 2, P - 1, P) and push
     if (k >= 2) {
@@ -398,35 +414,12 @@ __device__ __forceinline__ bool fused_march(const MarchArgs &m, OutPop out_pop, 
           return pl[c0 + L::cy(i) * PW + L::cx(i)];
         };
         if constexpr (F64) {
-          // FP64: the oracle's operation order, velocity by velocity
-          C rho = 0, jx = 0, jy = 0, jz = 0;
-#pragma unroll
-          for (int i = 0; i < Q; ++i) {
-            rho += cur[i];
-            jx += (C)L::cx(i) * cur[i];
-            jy += (C)L::cy(i) * cur[i];
-            jz += (C)L::cz(i) * cur[i];
-          }
-          C sx = 0, sy = 0, sz = 0;
-#pragma unroll
-          for (int i = 1; i < Q; ++i) {
-            const C wp = (C)L::w(i) * psi_at(i);
-            sx += (C)L::cx(i) * wp;
-            sy += (C)L::cy(i) * wp;
-            sz += (C)L::cz(i) * wp;
-          }
-          const C gp = -G * p0[c0];
-          const C ux = (jx + tau * (gp * sx)) / rho, uy = (jy + tau * (gp * sy)) / rho,
-                  uz = (jz + tau * (gp * sz)) / rho;
-          const C uu = (C)1.5 * (ux * ux + uy * uy + uz * uz);
-#pragma unroll
-          for (int i = 0; i < Q; ++i) {
-            const C cu = (C)L::cx(i) * ux + (C)L::cy(i) * uy + (C)L::cz(i) * uz;
-            const C feq = (C)L::w(i) * rho * ((C)1 + (C)3 * cu + (C)4.5 * cu * cu - uu);
-            C fs = cur[i] - (cur[i] - feq) / tau;
-            if (site) fs += L::w(i) * dmc;
-            *dst(i) = S::store(fs);
-          }
+          auto f = [&](int i) { return cur[i]; };
+          auto put = [&](auto ic, C v) { *dst(decltype(ic)::value) = S::store(v); };
+          if (site)
+            collide_f64<LAT, true>(relax, f, Rcur, p0[c0], psi_at, put, dmc);
+          else
+            collide_f64<LAT, false>(relax, f, Rcur, p0[c0], psi_at, put, 0.0);
         } else {
           // FP32 on offsets g_i = f_i - w_i rho_ref: with R = sum g (so that
           // rho = rho_ref + R) the equilibrium offset is
@@ -510,8 +503,10 @@ __device__ __forceinline__ bool fused_march(const MarchArgs &m, OutPop out_pop, 
       }
     }
     if constexpr (F64) {
+      if (active && k >= 1 && k + 1 < NPL) {
 #pragma unroll
-      for (int i = 0; i < Q; ++i) cur[i] = nxt[i];
+        for (int i = 0; i < Q; ++i) cur[i] = S::load(mainb[(i * BY + ty) * BX + tx]);
+      }
     } else {
 #pragma unroll
       for (int k2 = 0; k2 < L::NP; ++k2) cur2[k2] = nxt2[k2];
@@ -567,9 +562,10 @@ __device__ __forceinline__ MarchArgs march_args_of(const FusedMaps &tm, const St
 // One launch per time step: CTA (item) = BX x BY tile tt and z chunk zc,
 // item = zc * tiles + tt, so the CTAs resident together cover neighbouring
 // columns at the same planes (their halo rows meet in L2).
-// 256-thread tiles are register-limited to 3 CTAs per SM, the larger ones run one
+// 256-thread tiles are register-limited to 3 CTAs per SM (FP64: shared
+// memory holds 2, which leaves 128 registers), the larger ones run one
 template <int LAT, int ST, int BX, int BY, int NS>
-__global__ void __launch_bounds__(BX *BY, BX *BY <= 256 ? 3 : 1)
+__global__ void __launch_bounds__(BX *BY, BX *BY <= 256 ? (ST == ST_F64 ? 2 : 3) : 1)
     fused_step_kernel(const __grid_constant__ FusedMaps tm, const StepArgs a, const int tiles_x,
                       const int tiles_y, const int zlen) {
   using T = typename Storage<ST>::T;
