@@ -580,6 +580,7 @@ lbm_status lbm_step(lbm_ctx *c, int64_t nsteps) {
   a.G = c->cfg.G;
   a.rho0 = c->cfg.rho0;
   a.rho_ref = c->cfg.rho_ref;
+  a.relax = make_relax(c->cfg.tau, c->cfg.G, c->cfg.rho0);
   a.nsites = c->ninj;
   a.site_x = static_cast<const int32_t *>(c->d_sx.p);
   a.site_y = static_cast<const int32_t *>(c->d_sy.p);

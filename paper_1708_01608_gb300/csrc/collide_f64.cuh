@@ -20,6 +20,7 @@
 // density is the psi phase's sum.
 #pragma once
 
+#include "internal.h"
 #include "lattice.cuh"
 
 namespace sclbm {
@@ -68,8 +69,8 @@ __device__ __forceinline__ double psi_f64(double rho, double rho0, double inv_rh
 // Density of one cell from its Q values, in two chains (half the latency of
 // one; the owner and a neighbour's halo thread use the same order)
 template <int Q, class Ld>
-__device__ __forceinline__ double rho_f64(Ld ld) {
-  double a = ld(0), b = ld(1);
+__device__ __forceinline__ auto rho_f64(Ld ld) {
+  auto a = ld(0), b = ld(1);
 #pragma unroll
   for (int i = 2; i + 1 < Q; i += 2) {
     a += ld(i);
@@ -79,70 +80,62 @@ __device__ __forceinline__ double rho_f64(Ld ld) {
   return a + b;
 }
 
-template <int LAT>
-struct RelaxF64 {
-  static constexpr double R = LAT == D3Q19 ? 2.0 : 4.0;     // axis weight / edge weight
-  static constexpr double R0 = LAT == D3Q19 ? 12.0 : 16.0;  // rest weight / edge weight
-  double om1, fG, wK, cB;
-  __device__ __forceinline__ RelaxF64(double tau, double G) {
-    const double omega = 1.0 / tau, w = 1.0 / 36.0;
-    om1 = 1.0 - omega;
-    fG = -tau * G * w;
-    wK = omega * w;
-    cB = 3.0 * omega * w;
-  }
+// Relaxation constants; w is the edge weight 1/36.
+template <int LAT, class T>
+struct RelaxK {
+  static constexpr T R = LAT == D3Q19 ? 2 : 4;     // axis weight / edge weight
+  static constexpr T R0 = LAT == D3Q19 ? 12 : 16;  // rest weight / edge weight
+  T om1, wK, cB;
+  __device__ __forceinline__ RelaxK(T om1_, T wK_, T cB_) : om1(om1_), wK(wK_), cB(cB_) {}
 };
 
-template <int CC>
-__device__ __forceinline__ double cacc_d(double acc, double v) {
+template <int CC, class T>
+__device__ __forceinline__ T cacc_t(T acc, T v) {
   if constexpr (CC > 0) return acc + v;
   else if constexpr (CC < 0) return acc - v;
   else return acc;
 }
 
-// f(i): the cell's populations, rho their sum, psi0 and psi(i) the
-// pseudopotential here and at x + c_i; put(i, v) takes the collided
-// population (integral_constant i).  SITE adds w_i dm to every population.
-template <int LAT, bool SITE, class F, class Psi, class Put>
-__device__ __forceinline__ void collide_f64(const RelaxF64<LAT> &q, F f, double rho, double psi0,
-                                            Psi psi, Put put, double dm) {
+// sum_i w_i q(i) c_i / w over opposite pairs, q(i) given as the difference
+// dq(i) = q(i) - q(opp i) of a representative
+template <int LAT, bool WEIGHTED, class T, class Dq>
+__device__ __forceinline__ void pair_moments(Dq dq, T (&m)[3]) {
   using L = Lattice<LAT>;
-  constexpr double R = RelaxF64<LAT>::R, R0 = RelaxF64<LAT>::R0;
   // -0 is the additive identity, so a first term is no addition
-  double j[3] = {-0.0, -0.0, -0.0}, ax[3] = {0.0, 0.0, 0.0}, ed[3] = {-0.0, -0.0, -0.0};
+  T ax[3] = {0, 0, 0}, ed[3] = {(T)-0.0, (T)-0.0, (T)-0.0};
   static_for<L::NP>([&](auto kc) {
-    constexpr int i = L::rep(decltype(kc)::value), o = L::opp(i);
+    constexpr int i = L::rep(decltype(kc)::value);
     constexpr int cx = L::cx(i), cy = L::cy(i), cz = L::cz(i);
-    constexpr bool axis = cx * cx + cy * cy + cz * cz == 1;
-    const double d = f(i) - f(o), dp = psi(i) - psi(o);
-    j[0] = cacc_d<cx>(j[0], d);
-    j[1] = cacc_d<cy>(j[1], d);
-    j[2] = cacc_d<cz>(j[2], d);
-    if constexpr (axis) {
+    const T d = dq(std::integral_constant<int, i>{});
+    if constexpr (WEIGHTED && cx * cx + cy * cy + cz * cz == 1) {
       static_assert(cx + cy + cz == 1, "axis representatives point along +a");
-      ax[cx ? 0 : (cy ? 1 : 2)] = dp;
+      ax[cx ? 0 : (cy ? 1 : 2)] = d;
     } else {
-      ed[0] = cacc_d<cx>(ed[0], dp);
-      ed[1] = cacc_d<cy>(ed[1], dp);
-      ed[2] = cacc_d<cz>(ed[2], dp);
+      ed[0] = cacc_t<cx>(ed[0], d);
+      ed[1] = cacc_t<cy>(ed[1], d);
+      ed[2] = cacc_t<cz>(ed[2], d);
     }
   });
-  const double gp = q.fG * psi0, ir = 1.5 * __drcp_rn(rho);
-  double v[3], B[3], Q[3], s = -0.0;
+#pragma unroll
+  for (int a = 0; a < 3; ++a)
+    m[a] = WEIGHTED && (a != 1 || L::HAS_Y) ? fma(RelaxK<LAT, T>::R, ax[a], ed[a]) : ed[a];
+}
+
+// The relaxed populations of a cell: f(i) its populations, rho their sum,
+// v = 1.5 u, B = 3 omega w rho u; out(integral_constant i, value).
+template <int LAT, class T, class F, class Out>
+__device__ __forceinline__ void relax_pairs(const RelaxK<LAT, T> &q, F f, T rho, const T (&v)[3],
+                                            const T (&B)[3], Out out) {
+  using L = Lattice<LAT>;
+  constexpr T R = RelaxK<LAT, T>::R, R0 = RelaxK<LAT, T>::R0;
+  T Q[3], s = (T)-0.0;
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
     if (a == 1 && !L::HAS_Y) continue;
-    const double m = fma(gp, fma(R, ax[a], ed[a]), j[a]);
-    v[a] = m * ir;
-    B[a] = q.cB * m;
     Q[a] = B[a] * v[a];
     s += Q[a];
   }
-  const double K = fma(s, -1.0 / 3.0, q.wK * rho);
-  auto out = [&](auto ic, double x) {
-    constexpr int i = decltype(ic)::value;
-    put(ic, SITE ? x + L::w(i) * dm : x);
-  };
+  const T K = fma(s, (T)(-1.0 / 3.0), q.wK * rho);
   out(std::integral_constant<int, 0>{}, fma(q.om1, f(0), R0 * K));
   static_for<L::NP>([&](auto kc) {
     constexpr int i = L::rep(decltype(kc)::value), o = L::opp(i);
@@ -150,19 +143,46 @@ __device__ __forceinline__ void collide_f64(const RelaxF64<LAT> &q, F f, double 
     constexpr int c[3] = {cx, cy, cz};
     constexpr int a = cx ? 0 : (cy ? 1 : 2);
     if constexpr (cx * cx + cy * cy + cz * cz == 1) {
-      const double A = R * (K + Q[a]);
+      const T A = R * (K + Q[a]);
       out(std::integral_constant<int, i>{}, fma(R, B[a], fma(q.om1, f(i), A)));
       out(std::integral_constant<int, o>{}, fma(-R, B[a], fma(q.om1, f(o), A)));
     } else {
       constexpr int b = cz ? 2 : 1;
-      const double D = (K + Q[a]) + Q[b], v2 = v[b] + v[b];
-      const double A = c[a] * c[b] > 0 ? fma(B[a], v2, D) : fma(-B[a], v2, D);
+      const T D = (K + Q[a]) + Q[b], v2 = v[b] + v[b];
+      const T A = c[a] * c[b] > 0 ? fma(B[a], v2, D) : fma(-B[a], v2, D);
       // c_a B_a + c_b B_b up to the sign of c_a
-      const double t = c[a] * c[b] > 0 ? B[a] + B[b] : B[a] - B[b];
-      const double hi = fma(q.om1, f(i), A), ho = fma(q.om1, f(o), A);
+      const T t = c[a] * c[b] > 0 ? B[a] + B[b] : B[a] - B[b];
+      const T hi = fma(q.om1, f(i), A), ho = fma(q.om1, f(o), A);
       out(std::integral_constant<int, i>{}, c[a] > 0 ? hi + t : hi - t);
       out(std::integral_constant<int, o>{}, c[a] > 0 ? ho - t : ho + t);
     }
+  });
+}
+
+// The FP64 collision of one cell.  f(i): its populations, rho their sum,
+// psi0 and psi(i) the pseudopotential here and at x + c_i, fG = -tau G w;
+// put(i, v) takes the collided population (integral_constant i).  SITE adds
+// w_i dm to every population.
+template <int LAT, bool SITE, class F, class Psi, class Put>
+__device__ __forceinline__ void collide_f64(const RelaxK<LAT, double> &q, double fG, F f,
+                                            double rho, double psi0, Psi psi, Put put, double dm) {
+  using L = Lattice<LAT>;
+  double j[3], s[3];
+  pair_moments<LAT, false, double>(
+      [&](auto ic) { return f(decltype(ic)::value) - f(L::opp(decltype(ic)::value)); }, j);
+  pair_moments<LAT, true, double>(
+      [&](auto ic) { return psi(decltype(ic)::value) - psi(L::opp(decltype(ic)::value)); }, s);
+  const double gp = fG * psi0, ir = 1.5 * __drcp_rn(rho);
+  double v[3], B[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    if (a == 1 && !L::HAS_Y) continue;
+    const double m = fma(gp, s[a], j[a]);
+    v[a] = m * ir;
+    B[a] = q.cB * m;
+  }
+  relax_pairs<LAT, double>(q, f, rho, v, B, [&](auto ic, double x) {
+    put(ic, SITE ? x + L::w(decltype(ic)::value) * dm : x);
   });
 }
 

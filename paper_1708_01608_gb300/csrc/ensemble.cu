@@ -67,8 +67,6 @@ __device__ __forceinline__ MarchArgs ens_march_args(const EnsDomain &D, const in
   m.NY = 1;
   m.NZ = D.NZ;
   m.px = D.px;
-  m.tau = D.tau;
-  m.G = D.G;
   m.rho0 = D.rho0;
   m.tau_f = D.tau_f;
   m.omega_f = D.omega_f;

@@ -12,6 +12,17 @@ namespace sclbm {
 // store a message for lbm_last_error() and return st
 lbm_status set_error(lbm_status st, const char *msg);
 
+// Constants of the FP64 collision (collide_f64.cuh), formed on the host: a
+// division per thread would cost a tenth of a small lattice's step.
+struct RelaxArgs {
+  double om1, wK, cB;   // 1 - omega, omega w, 3 omega w (w = 1/36)
+  double fG, inv_rho0;  // -tau G w, 1/rho0
+};
+inline RelaxArgs make_relax(double tau, double G, double rho0) {
+  const double omega = 1.0 / tau, w = 1.0 / 36.0;
+  return RelaxArgs{1.0 - omega, omega * w, 3.0 * omega * w, -tau * G * w, 1.0 / rho0};
+}
+
 // Everything a step kernel needs.  Cells are addressed in the kernels'
 // three-dimensional view (D2Q9 on (nx, 1, ny)); the population arrays are
 // f[i][z][y][x] with a row pitch px >= NX (elements), planes of px*NY and
@@ -22,6 +33,7 @@ struct StepArgs {
   void *fout;
   int64_t NX, NY, NZ, px;
   double tau, G, rho0, rho_ref;
+  RelaxArgs relax;
   // the same constants in FP32 (the FP32-arithmetic kernels use no FP64)
   float tau_f, omega_f, G_f, rho0_f, inv_rho0_f, rho_ref_f;
   // base of every population block of fout (push destinations)

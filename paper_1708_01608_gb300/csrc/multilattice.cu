@@ -14,10 +14,10 @@
 // (u_s = u' where the lattice is empty: f_eq is 0 there).  eta_m(k, l) = 0
 // merges lattice l into k (f_k += f_l, f_l = 0) and removes their coupling.
 //
-// GB300 form: two passes per step (psi of every lattice into an FP64/FP32
-// field, then collide and push every lattice of a cell in one thread),
-// populations f[s][i][z][y][x] unpadded, plain values (no offset), FP64 or
-// FP32.  The FP64 form keeps the oracle's operation order.  The blowing
+// GB300 form: one launch per step for D2Q9 (psi of a tile and its halo in
+// shared memory), psi into a field first for D3Q19; one thread per (cell,
+// lattice); populations f[s][i][z][y][x] unpadded, plain values (no offset),
+// FP64 or FP32.  The blowing
 // agent of site k deposits w_i dm into lattice k (one thread walks the
 // sites in order after the step, on the pushed populations at x_k + c_i).
 #include <algorithm>
@@ -26,6 +26,7 @@
 #include <string>
 #include <vector>
 
+#include "collide_f64.cuh"
 #include "internal.h"
 #include "lattice.cuh"
 #include "lbm.h"
@@ -36,14 +37,20 @@ namespace {
 
 constexpr int ML_MAX = 8;  // lattices: the fluid and up to seven bubbles
 constexpr int TPB = 256;
+constexpr int ML_TPB = 256;  // threads of a step CTA at most: two or three CTAs per SM
 
+// (T: the constants in the arithmetic type of the kernel.  Converting them per
+// thread would run on the FP64 pipe: with nl^2 couplings per cell that alone
+// was a tenth of an FP32 step.)
+template <class T>
 struct MlArgs {
   const void *fin;
   void *fout;
   int64_t NX, NY, NZ;  // view extents (D2Q9 on (nx, 1, ny))
   int nl;
-  double tau, rho0;
-  double Gm[ML_MAX * ML_MAX];
+  T rho0, inv_rho0;
+  T om1, wK, cB, fG;  // RelaxArgs
+  T Gm[ML_MAX * ML_MAX];
 };
 
 inline int nblocks(int64_t n) {
@@ -60,101 +67,175 @@ __device__ __forceinline__ double ml_psi(double rho, double rho0) {
 __device__ __forceinline__ float ml_psi(float rho, float rho0) {
   return rho0 * (1.0f - expf(-rho / rho0));
 }
+// the step kernels' psi, density and reciprocal
+__device__ __forceinline__ double ml_psi_fast(double rho, double rho0, double inv_rho0) {
+  return psi_f64(rho, rho0, inv_rho0);
+}
+__device__ __forceinline__ float ml_psi_fast(float rho, float rho0, float) {
+  return ml_psi(rho, rho0);
+}
+template <int Q, class T>
+__device__ __forceinline__ T ml_rho(const T *f, int64_t N) {
+  return rho_f64<Q>([&](int i) { return f[i * N]; });
+}
+__device__ __forceinline__ double ml_rcp(double v) { return __drcp_rn(v); }
+__device__ __forceinline__ float ml_rcp(float v) { return 1.0f / v; }
 
-// pass 1: psi of every lattice at every cell (density summed in velocity order)
+// What the step kernels need beside MlArgs: the work split (ml_tile).  A CTA
+// takes tx x tz cells of every lattice, one thread per (cell, lattice); on the
+// field form tz is 1 and a CTA row y, z comes from the grid.
+struct MlTile {
+  int tx, tz;       // cells of a CTA along x and along the view's z (D2Q9)
+  int threads, smem;
+  unsigned gx, gy;  // grid
+  FastDiv fcells, ftx, fpw, fny;  // by tx tz, tx, tx + 2, NY
+};
+
+// psi of every lattice into a field, one thread per (cell, lattice): D3Q19,
+// where a tile's one-cell halo would cost as much psi as the tile itself
 template <int LAT, class T>
-__global__ void __launch_bounds__(TPB) k_ml_psi(const MlArgs a, T *psi) {
+__global__ void __launch_bounds__(TPB) k_ml_psi(const MlArgs<T> a, T *psi) {
   using L = Lattice<LAT>;
   const int64_t N = a.NX * a.NY * a.NZ;
   const T *f = static_cast<const T *>(a.fin);
-  const T rho0 = (T)a.rho0;
+  const T rho0 = a.rho0, inv_rho0 = a.inv_rho0;
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const int s = blockIdx.y;
   for (int64_t k = blockIdx.x * (int64_t)TPB + threadIdx.x; k < N; k += (int64_t)gridDim.x * TPB)
-    for (int s = 0; s < a.nl; ++s) {
-      T r = 0;
-#pragma unroll
-      for (int i = 0; i < L::Q; ++i) r += f[((int64_t)s * L::Q + i) * N + k];
-      psi[(int64_t)s * N + k] = ml_psi(r, rho0);
-    }
+    psi[(int64_t)s * N + k] =
+        ml_psi_fast(ml_rho<L::Q>(f + (int64_t)s * L::Q * N + k, N), rho0, inv_rho0);
 }
 
-// pass 2: moments, common velocity, forces, BGK and push of every lattice
-// (the oracle's operation order: the force of lattice s sums over t and i
-// jointly, F_s = -psi_s sum, u_s = u' + tau F_s / rho_s where rho_s != 0)
-template <int LAT, class T>
-__global__ void __launch_bounds__(TPB) k_ml_collide(const MlArgs a, const T *psi) {
+// One step of every lattice.  In small lattices (104^2 of the bubble-size
+// sweep: 71 cells per SM) the FP64 pipe is the bound only if every SM has
+// work, so a CTA holds one thread per (cell, lattice) and ml_tile picks the
+// tile that spreads the cells evenly over the SMs; the per-lattice parts
+// (density, momentum, psi gradient, relaxation) run side by side and meet in
+// shared memory for the two sums over lattices.  Operations follow
+// collide_f64.cuh.  Us per step with three lattices, a launch of one thread
+// per cell for psi and one for the collision of all lattices (844 FP64
+// instructions per cell, 43 CTAs at 104^2) against this form: FP64 104^2 96.9
+// / 11.8, 500^2 698 / 208, D3Q19 64x64x48 912 / 239; FP32 104^2 16.4 / 3.7,
+// 1000^2 161 / 118, 64x64x48 66.6 / 27.2.
+//
+// FIELD: psi comes from k_ml_psi (D3Q19).  Otherwise (D2Q9) the CTA forms it
+// for its tile and a one-cell halo in shared memory, one launch per step.
+template <int LAT, class T, bool FIELD>
+__global__ void __launch_bounds__(ML_TPB, sizeof(T) == 8 ? 2 : 3) k_ml_step(const MlArgs<T> a, const MlTile tl,
+                                                 const T *psi_field) {
   using L = Lattice<LAT>;
   constexpr int Q = L::Q;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int nl = a.nl, cells = tl.tx * tl.tz;
+  const int PW = tl.tx + 2, PC = FIELD ? 0 : PW * (tl.tz + 2);
+  T *sG = reinterpret_cast<T *>(smem_raw);  // coupling matrix
+  T *mom = sG + ML_MAX * ML_MAX;            // [lattice][rho, j (3), S (3)][cell]
+  T *psis = mom + nl * 7 * cells;           // [lattice][PC]
+  const int NX = (int)a.NX, NY = (int)a.NY, NZ = (int)a.NZ;
   const int64_t N = a.NX * a.NY * a.NZ;
   const T *f = static_cast<const T *>(a.fin);
-  T *g = static_cast<T *>(a.fout);
-  const int NX = (int)a.NX, NY = (int)a.NY, NZ = (int)a.NZ;
-  const T tau = (T)a.tau;
-  for (int64_t k = blockIdx.x * (int64_t)TPB + threadIdx.x; k < N;
-       k += (int64_t)gridDim.x * TPB) {
-    const int x = (int)(k % NX), y = (int)((k / NX) % NY), z = (int)(k / ((int64_t)NX * NY));
-    // neighbour cells x + c_i, periodic
-    int64_t nbk[Q];
-#pragma unroll
-    for (int i = 0; i < Q; ++i)
-      nbk[i] = ((int64_t)wrapv(z + L::cz(i), NZ) * NY + wrapv(y + L::cy(i), NY)) * NX +
-               wrapv(x + L::cx(i), NX);
-    T rho[ML_MAX];
-    T rt = 0, jtx = 0, jty = 0, jtz = 0;
-    for (int s = 0; s < a.nl; ++s) {
-      T r = 0, ax = 0, ay = 0, az = 0;
+  const int tid = threadIdx.x, x0 = blockIdx.y * tl.tx;
+  for (int k = tid; k < ML_MAX * ML_MAX; k += blockDim.x) sG[k] = a.Gm[k];
+  const RelaxK<LAT, T> relax(a.om1, a.wK, a.cB);
+  const T rho0 = a.rho0, inv_rho0 = a.inv_rho0;
+  const int s = (int)fdiv((uint32_t)tid, tl.fcells, (uint32_t)cells), c = tid - s * cells;
+  const int cz_ = FIELD ? 0 : (int)fdiv((uint32_t)c, tl.ftx, (uint32_t)tl.tx);
+  const int cx_ = c - cz_ * tl.tx;
+  const int x = x0 + cx_;
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+
+  const T *fs = f + (int64_t)s * Q * N;
+  const uint32_t rows = FIELD ? (uint32_t)(a.NY * a.NZ) : 1u;
+  for (uint32_t row = FIELD ? blockIdx.x : 0; row < rows; row += gridDim.x) {
+    const int z0 = FIELD ? (int)fdiv(row, tl.fny, (uint32_t)NY) : (int)blockIdx.x * tl.tz;
+    const int y = FIELD ? (int)(row - (uint32_t)z0 * (uint32_t)NY) : 0, z = z0 + cz_;
+    const bool on = s < nl && x < NX && z < NZ;
+    if constexpr (!FIELD) {
+      if (s < nl)
+        for (int r = c; r < PC; r += cells) {
+          const int rz = (int)fdiv((uint32_t)r, tl.fpw, (uint32_t)PW);
+          // cells past a ragged tile's halo are not read by anyone
+          const int hx = x0 + r - rz * PW - 1, hz = z0 + rz - 1;
+          if (hx > NX || hz > NZ) continue;
+          const uint32_t k = (uint32_t)wrapv(hz, NZ) * (uint32_t)NX + (uint32_t)wrapv(hx, NX);
+          psis[s * PC + r] = ml_psi_fast(ml_rho<Q>(fs + k, N), rho0, inv_rho0);
+        }
+      __syncthreads();
+    }
+    T fi[Q], rho = 0, psi0 = 0;
+    uint32_t nb[Q];  // a lattice has fewer than 2^32 cells (lbm_ml_create)
+    if (on) {
+      const int xs[3] = {wrapv(x - 1, NX), x, wrapv(x + 1, NX)};
+      const int ys[3] = {wrapv(y - 1, NY), y, wrapv(y + 1, NY)};
+      const int zs[3] = {wrapv(z - 1, NZ), z, wrapv(z + 1, NZ)};
 #pragma unroll
       for (int i = 0; i < Q; ++i) {
-        const T v = f[((int64_t)s * Q + i) * N + k];
-        r += v;
-        ax += v * (T)L::cx(i);
-        ay += v * (T)L::cy(i);
-        az += v * (T)L::cz(i);
+        nb[i] = ((uint32_t)zs[L::cz(i) + 1] * (uint32_t)NY + (uint32_t)ys[L::cy(i) + 1]) *
+                    (uint32_t)NX + (uint32_t)xs[L::cx(i) + 1];
       }
-      rho[s] = r;
-      rt += r;
-      jtx += ax;
-      jty += ay;
-      jtz += az;
-    }
-    const T upx = jtx / rt, upy = jty / rt, upz = jtz / rt;
-    for (int s = 0; s < a.nl; ++s) {
-      T ax = 0, ay = 0, az = 0;
-      for (int t = 0; t < a.nl; ++t) {
-        const T G = (T)a.Gm[s * ML_MAX + t];
 #pragma unroll
-        for (int i = 1; i < Q; ++i) {
-          const T v = G * (T)L::w(i) * psi[(int64_t)t * N + nbk[i]];
-          ax += v * (T)L::cx(i);
-          ay += v * (T)L::cy(i);
-          az += v * (T)L::cz(i);
+      for (int i = 0; i < Q; ++i) fi[i] = fs[i * N + nb[0]];
+      rho = rho_f64<Q>([&](int i) { return fi[i]; });
+      const T *pf = FIELD ? psi_field + (int64_t)s * N
+                          : psis + s * PC + (cz_ + 1) * PW + cx_ + 1;
+      auto psi = [&](int i) -> T {
+        return FIELD ? pf[nb[i]] : pf[L::cz(i) * PW + L::cx(i)];
+      };
+      psi0 = psi(0);
+      T j[3], S[3];
+      pair_moments<LAT, false, T>(
+          [&](auto ic) { return fi[decltype(ic)::value] - fi[L::opp(decltype(ic)::value)]; }, j);
+      pair_moments<LAT, true, T>(
+          [&](auto ic) { return psi(decltype(ic)::value) - psi(L::opp(decltype(ic)::value)); }, S);
+      T *m = mom + s * 7 * cells + c;
+      m[0] = rho;
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        m[(1 + d) * cells] = j[d];
+        m[(4 + d) * cells] = S[d];
+      }
+    }
+    __syncthreads();
+    if (on) {
+      // common velocity sum j / sum rho and the force sum over lattices
+      T rt = 0, jt[3] = {0, 0, 0}, A[3] = {0, 0, 0};
+      for (int t = 0; t < nl; ++t) {
+        const T *m = mom + t * 7 * cells + c;
+        const T g = sG[s * ML_MAX + t];
+        rt += m[0];
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+          if (d == 1 && !L::HAS_Y) continue;
+          jt[d] += m[(1 + d) * cells];
+          A[d] = fma(g, m[(4 + d) * cells], A[d]);
         }
       }
-      const T ps = psi[(int64_t)s * N + k];
-      const T Fx = -ps * ax, Fy = -ps * ay, Fz = -ps * az;
-      const T r = rho[s];
-      T ux = upx, uy = upy, uz = upz;
-      if (r != (T)0) {
-        ux += tau * Fx / r;
-        uy += tau * Fy / r;
-        uz += tau * Fz / r;
-      }
-      const T uu = ux * ux + uy * uy + uz * uz;
+      const T ir = ml_rcp(rt);
+      // u_s = u' + tau F_s / rho_s where the lattice is not empty (fG: -tau w)
+      const T h = rho != (T)0 ? a.fG * psi0 * ml_rcp(rho) : (T)0;
+      T v[3], B[3];
 #pragma unroll
-      for (int i = 0; i < Q; ++i) {
-        const T cu = (T)L::cx(i) * ux + (T)L::cy(i) * uy + (T)L::cz(i) * uz;
-        const T feq =
-            (T)L::w(i) * r * ((T)1 + (T)3 * cu + (T)4.5 * cu * cu - (T)1.5 * uu);
-        const T fi = f[((int64_t)s * Q + i) * N + k];
-        g[((int64_t)s * Q + i) * N + nbk[i]] = fi - (fi - feq) / tau;
+      for (int d = 0; d < 3; ++d) {
+        if (d == 1 && !L::HAS_Y) continue;
+        const T u = fma(h, A[d], jt[d] * ir);
+        v[d] = (T)1.5 * u;
+        B[d] = relax.cB * (rho * u);
       }
+      T *g = static_cast<T *>(a.fout) + (int64_t)s * Q * N;
+      relax_pairs<LAT, T>(
+          relax, [&](int i) { return fi[i]; }, rho, v, B,
+          [&](auto ic, T val) { g[decltype(ic)::value * N + nb[decltype(ic)::value]] = val; });
     }
+    if (FIELD) __syncthreads();  // the moments are read before the next row writes them
   }
 }
 
 // the blowing agent, site by site in order (one thread): dm = min(rate,
 // budget) into lattice site_lat[m] at the pushed destinations x_m + c_i
 template <int LAT, class T>
-__global__ void k_ml_inject(const MlArgs a, int n, const int32_t *sx, const int32_t *sy,
+__global__ void k_ml_inject(const MlArgs<T> a, int n, const int32_t *sx, const int32_t *sy,
                             const int32_t *sz, const int32_t *slat, const double *rate,
                             double *budget) {
   using L = Lattice<LAT>;
@@ -192,12 +273,11 @@ __global__ void __launch_bounds__(TPB) k_ml_merge(T *f, int64_t QN, int k, int l
 // pressure of the coupled lattices, p = rho_total/3 + 1/6 sum_s sum_t
 // Gm[s][t] psi_s psi_t (p may be null)
 template <int LAT, class T>
-__global__ void __launch_bounds__(TPB) k_ml_fields(const MlArgs a, double *rho_out, double *p) {
+__global__ void __launch_bounds__(64) k_ml_fields(const MlArgs<double> a, double *rho_out, double *p) {
   using L = Lattice<LAT>;
   const int64_t N = a.NX * a.NY * a.NZ;
   const T *f = static_cast<const T *>(a.fin);
-  for (int64_t k = blockIdx.x * (int64_t)TPB + threadIdx.x; k < N;
-       k += (int64_t)gridDim.x * TPB) {
+  for (int64_t k = blockIdx.x * (int64_t)64 + threadIdx.x; k < N; k += (int64_t)gridDim.x * 64) {
     double rho[ML_MAX];
     double rt = 0.0;
     for (int s = 0; s < a.nl; ++s) {
@@ -209,10 +289,10 @@ __global__ void __launch_bounds__(TPB) k_ml_fields(const MlArgs a, double *rho_o
       if (rho_out) rho_out[(int64_t)s * N + k] = r;
     }
     if (p) {
-      double e = 0.0;
+      double e = 0.0, ps[ML_MAX];
+      for (int s = 0; s < a.nl; ++s) ps[s] = ml_psi(rho[s], a.rho0);
       for (int s = 0; s < a.nl; ++s)
-        for (int t = 0; t < a.nl; ++t)
-          e += a.Gm[s * ML_MAX + t] * ml_psi(rho[s], a.rho0) * ml_psi(rho[t], a.rho0);
+        for (int t = 0; t < a.nl; ++t) e += a.Gm[s * ML_MAX + t] * ps[s] * ps[t];
       p[k] = rt / 3.0 + e / 6.0;
     }
   }
@@ -258,6 +338,7 @@ struct lbm_ml_ctx {
   int32_t *d_site = nullptr;  // x, y, z, lattice per site (view coordinates)
   int32_t nsites = 0;
   std::vector<int32_t> site_xyz;
+  MlTile tile{};
   int cur = 0;
   bool seeded = false;
   int64_t steps = 0;
@@ -336,18 +417,86 @@ struct MlTemp {
   }
 };
 
-MlArgs ml_args(const lbm_ml_ctx *c) {
-  MlArgs a{};
+template <class T>
+MlArgs<T> ml_args(const lbm_ml_ctx *c) {
+  MlArgs<T> a{};
   a.fin = c->cur == 0 ? c->fA : c->fB;
   a.fout = c->cur == 0 ? c->fB : c->fA;
   a.NX = c->v.NX;
   a.NY = c->v.NY;
   a.NZ = c->v.NZ;
   a.nl = c->nl;
-  a.tau = c->cfg.tau;
-  a.rho0 = c->cfg.rho0;
-  std::memcpy(a.Gm, c->Gm, sizeof(a.Gm));
+  const RelaxArgs r = make_relax(c->cfg.tau, 1.0, c->cfg.rho0);  // the couplings are in Gm
+  a.rho0 = (T)c->cfg.rho0;
+  a.inv_rho0 = (T)r.inv_rho0;
+  a.om1 = (T)r.om1;
+  a.wK = (T)r.wK;
+  a.cB = (T)r.cB;
+  a.fG = (T)r.fG;
+  for (int k = 0; k < ML_MAX * ML_MAX; ++k) a.Gm[k] = (T)c->Gm[k];
   return a;
+}
+
+// launched as a programmatic dependent of the previous kernel in the stream
+template <class... P, class... A>
+void ml_launch(const lbm_ml_ctx *c, dim3 grid, int threads, int smem, void (*k)(P...), A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = (size_t)smem;
+  cfg.stream = c->s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, k, args...);  // the error stays for cudaGetLastError
+}
+
+// The tile of the step kernel.  D2Q9: the tx x tz with the least work on the
+// busiest SM, a cell counting 5 (collision) and a halo position 1 (psi), plus
+// 40 for the launch's fixed latency per CTA.  D3Q19: 64 cells of a row (32
+// from five lattices on).
+MlTile ml_tile(int lat, int nl, int ts, int64_t NX, int64_t NY, int64_t NZ, int nsm) {
+  MlTile best{};
+  auto fill = [&](MlTile &t) {
+    const int cells = t.tx * t.tz;
+    t.threads = (cells * nl + 31) / 32 * 32;
+    t.fcells = make_fastdiv((uint32_t)cells);
+    t.ftx = make_fastdiv((uint32_t)t.tx);
+    t.fpw = make_fastdiv((uint32_t)t.tx + 2);
+    t.fny = make_fastdiv((uint32_t)NY);
+    t.smem = ts * (ML_MAX * ML_MAX + nl * (7 * cells + (lat == D2Q9 ? (t.tx + 2) * (t.tz + 2) : 0)));
+  };
+  if (lat == D3Q19) {
+    best.tx = nl > 4 ? 32 : 64;
+    best.tz = 1;
+    best.gx = (unsigned)std::min<int64_t>(NY * NZ, 1 << 30);
+    best.gy = (unsigned)((NX + best.tx - 1) / best.tx);
+    fill(best);
+    return best;
+  }
+  double cost = 0;
+  for (int tx = 8; tx <= 64; tx += 8)
+    for (int tz = 1; tz <= 32; ++tz) {
+      MlTile t{};
+      t.tx = tx;
+      t.tz = tz;
+      fill(t);
+      const int64_t gx = (NZ + tz - 1) / tz, gy = (NX + tx - 1) / tx;
+      if (t.threads > ML_TPB || t.smem > 48 * 1024 || gy > 65535) continue;
+      // beyond a few tiles per SM rows of whole 128-byte lines
+      if (gx * gy > 4 * nsm && tx * ts < 128) continue;
+      t.gx = (unsigned)gx;
+      t.gy = (unsigned)gy;
+      const double w = (double)((gx * gy + nsm - 1) / nsm) *
+                       (5.0 * tx * tz + (double)(tx + 2) * (tz + 2) + 40.0);
+      if (best.tx == 0 || w < cost) {
+        cost = w;
+        best = t;
+      }
+    }
+  return best;
 }
 
 template <class Fn>
@@ -426,12 +575,23 @@ lbm_status lbm_ml_create(const lbm_ml_config *cfg, lbm_ml_ctx **out) {
   c->v.rho_ref = 0.0;
   view_prepare(c->v);
   c->N = c->v.NX * c->v.NY * c->v.NZ;
+  if (c->N > (int64_t)UINT32_MAX) {  // at least 96 bytes a cell: beyond the card's memory
+    delete c;
+    return ml_fail(LBM_ENOMEM, "device allocation failed");
+  }
   // coupling matrix of the reading above; eta_m = 1 for every pair
   for (int s = 0; s < c->nl; ++s)
     for (int t = 0; t < c->nl; ++t)
       c->Gm[s * ML_MAX + t] =
           (s == 0 && t == 0) ? cfg->G : ((s == 0 || t == 0) ? cfg->G_x : (s == t ? 0.0 : cfg->G_b));
   const size_t ts = c->f64 ? 8 : 4;
+  int dev = 0, nsm = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+    cudaGetLastError();  // the allocations below report a missing device
+    nsm = 1;
+  }
+  c->tile = ml_tile(c->lat, c->nl, (int)ts, c->v.NX, c->v.NY, c->v.NZ, nsm);
   c->lat_bytes = ts * (size_t)c->nl * c->Q * c->N;
   lbm_status st;
   auto bail = [&](lbm_status e) {
@@ -440,7 +600,8 @@ lbm_status lbm_ml_create(const lbm_ml_config *cfg, lbm_ml_ctx **out) {
   };
   if ((st = ml_alloc(c, &c->fA, c->lat_bytes)) != LBM_OK) return bail(st);
   if ((st = ml_alloc(c, &c->fB, c->lat_bytes)) != LBM_OK) return bail(st);
-  if ((st = ml_alloc(c, &c->psi, ts * (size_t)c->nl * c->N)) != LBM_OK) return bail(st);
+  if (c->lat == D3Q19 && (st = ml_alloc(c, &c->psi, ts * (size_t)c->nl * c->N)) != LBM_OK)
+    return bail(st);
   if ((st = ml_alloc(c, (void **)&c->d_rho, sizeof(double) * (size_t)c->nl * c->N)) != LBM_OK)
     return bail(st);
   if ((st = ml_alloc(c, (void **)&c->d_p, sizeof(double) * (size_t)c->N)) != LBM_OK) return bail(st);
@@ -611,16 +772,24 @@ lbm_status lbm_ml_step(lbm_ml_ctx *c, int64_t nsteps) {
   if (nsteps < 0) return ml_fail(LBM_EINVAL, "nsteps < 0");
   if (!c->seeded) return ml_fail(LBM_ESTATE, "seed the lattices first");
   for (int64_t t = 0; t < nsteps; ++t) {
-    const MlArgs a = ml_args(c);
     cudaError_t e = ml_dispatch(c, [&](auto L, auto T) {
       using TT = decltype(T);
       constexpr int lat = decltype(L)::value;
-      k_ml_psi<lat, TT><<<nblocks(c->N), TPB, 0, c->s>>>(a, static_cast<TT *>(c->psi));
-      k_ml_collide<lat, TT><<<nblocks(c->N), TPB, 0, c->s>>>(a, static_cast<const TT *>(c->psi));
-      if (c->nsites > 0)
-        k_ml_inject<lat, TT><<<1, 32, 0, c->s>>>(a, c->nsites, c->d_site, c->d_site + ML_MAX,
-                                                  c->d_site + 2 * ML_MAX, c->d_site + 3 * ML_MAX,
-                                                  c->d_rate, c->d_budget);
+      const MlArgs<TT> a = ml_args<TT>(c);
+      TT *psi = static_cast<TT *>(c->psi);
+      if constexpr (lat == D3Q19)
+        ml_launch(c, dim3((unsigned)nblocks(c->N), (unsigned)c->nl), TPB, 0, k_ml_psi<lat, TT>, a,
+                  psi);
+      ml_launch(c, dim3(c->tile.gx, c->tile.gy), c->tile.threads, c->tile.smem,
+                  k_ml_step<lat, TT, lat == D3Q19>, a, c->tile, static_cast<const TT *>(psi));
+    });
+    if (e == cudaSuccess && c->nsites > 0) e = ml_dispatch(c, [&](auto L, auto T) {
+      using TT = decltype(T);
+      constexpr int lat = decltype(L)::value;
+      const MlArgs<TT> a = ml_args<TT>(c);
+      k_ml_inject<lat, TT><<<1, 32, 0, c->s>>>(a, c->nsites, c->d_site, c->d_site + ML_MAX,
+                                                c->d_site + 2 * ML_MAX, c->d_site + 3 * ML_MAX,
+                                                c->d_rate, c->d_budget);
     });
     if (e != cudaSuccess) {
       cudaGetLastError();
@@ -649,13 +818,20 @@ lbm_status lbm_ml_merge(lbm_ml_ctx *c, int32_t k, int32_t l) {
   return ml_sync(c);
 }
 
+// densities and pressure of the current state into d_rho and d_p (enqueued)
+static lbm_status ml_enqueue_fields(lbm_ml_ctx *c) {
+  const MlArgs<double> a = ml_args<double>(c);
+  MLCK(ml_dispatch(c, [&](auto L, auto T) {
+    k_ml_fields<decltype(L)::value, decltype(T)>
+        <<<(int)std::min<int64_t>((c->N + 63) / 64, 1 << 20), 64, 0, c->s>>>(a, c->d_rho, c->d_p);
+  }));
+  return LBM_OK;
+}
+
 lbm_status lbm_ml_fields(lbm_ml_ctx *c, double *rho, double *p) {
   if (!c) return ml_fail(LBM_EINVAL, "ctx is NULL");
   if (!c->seeded) return ml_fail(LBM_ESTATE, "seed the lattices first");
-  const MlArgs a = ml_args(c);
-  MLCK(ml_dispatch(c, [&](auto L, auto T) {
-    k_ml_fields<decltype(L)::value, decltype(T)><<<nblocks(c->N), TPB, 0, c->s>>>(a, c->d_rho, c->d_p);
-  }));
+  MLCKS(ml_enqueue_fields(c));
   if (rho)
     MLCK(cudaMemcpyAsync(rho, c->d_rho, sizeof(double) * (size_t)c->nl * c->N,
                          cudaMemcpyDeviceToHost, c->s));
@@ -698,7 +874,7 @@ lbm_status lbm_ml_run_until_rupture(lbm_ml_ctx *c, const int64_t *line, double r
     MLCKS(lbm_ml_step(c, n));
     t += n;
     // the film on the fluid lattice's density, with the coupled pressure
-    MLCKS(lbm_ml_fields(c, nullptr, nullptr));
+    MLCKS(ml_enqueue_fields(c));
     MLCK(diag_film_probe(c->v, c->d_rho, c->d_p, wr(x0, c->v.NX), wr(y0, c->v.NY), wr(z0, c->v.NZ),
                          e, ep, line[4], rho_mid, c->d_tmp, c->s));
     MLCK(cudaMemcpyAsync(h, c->d_tmp, sizeof(h), cudaMemcpyDeviceToHost, c->s));

@@ -77,7 +77,8 @@ struct FusedK {
 struct MarchArgs {
   int NX, NY, NZ;
   int64_t px;
-  double tau, G, rho0;  // FP64 arithmetic
+  double rho0;  // FP64 arithmetic
+  RelaxArgs relax;
   float tau_f, omega_f, G_f, rho0_f, inv_rho0_f, rho_ref_f;
   const FusedMaps *tm;
   int x0, y0, zs, ze;
@@ -179,9 +180,9 @@ __device__ __forceinline__ bool fused_march(const MarchArgs &m, OutPop out_pop, 
   const int64_t plane = m.px * NY;
 
   // constants in the arithmetic type (FP32 kernels execute no FP64 at all)
-  const C G = F64 ? (C)m.G : (C)m.G_f, tau = F64 ? (C)m.tau : (C)m.tau_f,
-          omega = F64 ? (C)(1.0 / m.tau) : (C)m.omega_f, rho0 = F64 ? (C)m.rho0 : (C)m.rho0_f,
-          inv_rho0 = F64 ? (C)(1.0 / m.rho0) : (C)m.inv_rho0_f;
+  const C G = (C)m.G_f, tau = (C)m.tau_f, omega = (C)m.omega_f,
+          rho0 = F64 ? (C)m.rho0 : (C)m.rho0_f,
+          inv_rho0 = F64 ? (C)m.relax.inv_rho0 : (C)m.inv_rho0_f;
   // offset storage: the staged values are g_i = f_i - w_i rho_ref
   const C rho_ref = S::OFFSET ? (C)m.rho_ref_f : (C)0;
 
@@ -315,7 +316,7 @@ __device__ __forceinline__ bool fused_march(const MarchArgs &m, OutPop out_pop, 
     c45[k2] = (C)4.5 * w * omega;
   }
 
-  [[maybe_unused]] const RelaxF64<LAT> relax(m.tau, m.G);
+  [[maybe_unused]] const RelaxK<LAT, double> relax(m.relax.om1, m.relax.wK, m.relax.cB);
 
   // two planes per iteration where registers allow (512-thread tiles): the
   // staged values then change register sets instead of being copied
@@ -417,9 +418,9 @@ __device__ __forceinline__ bool fused_march(const MarchArgs &m, OutPop out_pop, 
           auto f = [&](int i) { return cur[i]; };
           auto put = [&](auto ic, C v) { *dst(decltype(ic)::value) = S::store(v); };
           if (site)
-            collide_f64<LAT, true>(relax, f, Rcur, p0[c0], psi_at, put, dmc);
+            collide_f64<LAT, true>(relax, m.relax.fG, f, Rcur, p0[c0], psi_at, put, dmc);
           else
-            collide_f64<LAT, false>(relax, f, Rcur, p0[c0], psi_at, put, 0.0);
+            collide_f64<LAT, false>(relax, m.relax.fG, f, Rcur, p0[c0], psi_at, put, 0.0);
         } else {
           // FP32 on offsets g_i = f_i - w_i rho_ref: with R = sum g (so that
           // rho = rho_ref + R) the equilibrium offset is
@@ -530,8 +531,7 @@ __device__ __forceinline__ MarchArgs march_args_of(const FusedMaps &tm, const St
   m.NY = (int)a.NY;
   m.NZ = (int)a.NZ;
   m.px = a.px;
-  m.tau = a.tau;
-  m.G = a.G;
+  m.relax = a.relax;
   m.rho0 = a.rho0;
   m.tau_f = a.tau_f;
   m.omega_f = a.omega_f;

@@ -33,3 +33,36 @@ def test_fp64_step_over_the_range_of_psi(lbm, lat, ext, rho0):
     L.step(1)
     assert rel_err(L.read("f"), O.run(LAT[lat], f0, 1, 0.8, -5.0, rho0=rho0)) < 2e-14
     L.close()
+
+
+@pytest.mark.parametrize("lat,ext,nl", [
+    ("D2Q9", (1, 9, 1), 2), ("D2Q9", (8, 1, 1), 3), ("D2Q9", (65, 33, 1), 8),
+    ("D2Q9", (200, 131, 1), 4), ("D3Q19", (1, 5, 2), 1), ("D3Q19", (65, 3, 4), 4),
+    ("D3Q19", (33, 6, 5), 5), ("D3Q19", (64, 4, 3), 8)])
+@pytest.mark.parametrize("storage", ["f64", "f32"])
+def test_multi_lattice_step_tiles(lbm, lat, ext, nl, storage):
+    """One multi-lattice step at the edges of its tiles (one-cell extents,
+    ragged tiles, the lattice counts where the split changes), one lattice
+    empty.  A step rounds each population in about 60 terms of at most the
+    total density nl rho: 60 u nl, u = 1.1e-16 or 6e-8, relative to the
+    largest population (rho/3): 180 u nl, and FP32 also rounds the input."""
+    nx, ny, nz = ext
+    q = 19 if lat == "D3Q19" else 9
+    _, w = O.velocities(LAT[lat])
+    rng = np.random.default_rng(nl)
+    f0 = (w[None, :, None, None, None] * rng.uniform(0.1, 1.0, size=(nl, 1, nz, ny, nx))
+          * rng.uniform(0.9, 1.1, size=(nl, q, nz, ny, nx)))
+    if nl > 2:
+        f0[1] = 0.0
+    if storage == "f32":
+        f0 = f0.astype(np.float32).astype(np.float64)
+    M = lbm.MultiLattice(lat, nx, ny, nz, nl=nl, tau=0.9, G=-5.0, G_x=1.0, G_b=2.0,
+                         storage=storage)
+    M.write_f(f0)
+    M.step(1)
+    got = M.read_f()
+    want = O.ml_run(LAT[lat], f0, 1, 0.9, O.ml_coupling(nl, -5.0, 1.0, 2.0))
+    want = want[0] if isinstance(want, tuple) else want
+    u = 1.1e-16 if storage == "f64" else 6e-8
+    assert rel_err(got, want) < 180 * nl * u
+    M.close()
