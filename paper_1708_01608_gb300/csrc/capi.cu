@@ -361,7 +361,7 @@ lbm_status lbm_create(const lbm_config *cfg, lbm_ctx **out) {
     return bail(fail(LBM_ECUDA, "memset failed"));
   }
   if (c->kernel == LBM_KERNEL_FUSED) {
-    cudaError_t e = fused_make_plan(c->lat, c->st, cfg->tile, c->v.NX, c->v.NY, c->v.NZ, 0, &c->plan);
+    cudaError_t e = fused_make_plan(c->lat, c->st_step, cfg->tile, c->v.NX, c->v.NY, c->v.NZ, 0, &c->plan);
     if (e != cudaSuccess) {
       cudaGetLastError();
       if (cfg->kernel == LBM_KERNEL_FUSED)

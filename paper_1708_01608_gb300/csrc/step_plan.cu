@@ -36,8 +36,10 @@ static int fused_smem_bytes(int lat, int st, int tile, int xc) {
   if (xc == 2) {
     switch (st) {
       case ST_F32: return fused_x2_smem_f32(lat, tile);
-      case ST_F16: return fused_x2_smem_f16(lat, tile);
-      case ST_BF16: return fused_x2_smem_bf16(lat, tile);
+      case ST_F16:
+      case ST_F16R: return fused_x2_smem_f16(lat, tile);
+      case ST_BF16:
+      case ST_BF16R: return fused_x2_smem_bf16(lat, tile);
       default: return -1;
     }
   }
@@ -48,10 +50,116 @@ static int fused_smem_bytes(int lat, int st, int tile, int xc) {
   }
 }
 
+// The plan of a lattice whose tile the caller leaves open: the tile and chunk
+// count with the least time in this model (lbm_autotune measures instead).  A
+// CTA of a chunk of zl planes stages zl + 2 planes one after the other; a
+// plane takes max(floor, ns * cells * co), with co CTAs resident on an SM
+// (they share its issue slots and its memory path), and the step no less than
+// its populations take at the copy bandwidth.  The constants are fitted to the
+// times of every tile at 32^3 to 256^3 and 64^2 to 2000^2.  Every tile gives a
+// lattice the same bits.
+namespace {
+struct TileCost {
+  int tile;
+  // a plane in us: at least floor, ns per cell and resident CTA; with both
+  // lattices in L2, and beyond (one plane's HBM latency bounds a lone CTA)
+  float floor_l2, ns_l2, floor_hbm, ns_hbm;
+};
+// Us per step, former default (tile 1, at least 4 planes per chunk) / now.
+// FP32: 32^3 7.8 / 4.3, 64^3 11.8 / 9.9, 128^3 65.4 / 53.3, 256^3 464 / 394,
+// 512^3 4218 / 3178.  Tile 25 is for lattices it splits into one even wave
+// (128^3: 152 CTAs); in several waves it is the slower one (512^3: 3341).
+constexpr TileCost COST_F32[] = {{16, 1.1f, 2.45f, 1.35f, 3.03f}, {14, 1.1f, 2.45f, 1.35f, 3.03f},
+                                 {25, 1.1f, 2.45f, 1.35f, 3.03f}, {2, 0.5f, 4.0f, 1.35f, 6.0f}};
+// 16-bit: 32^3 7.9 / 4.4, 128^3 49.0 / 36.5, 256^3 379 / 238, 512^3 2848 / 1794
+constexpr TileCost COST_H16[] = {{24, 1.0f, 1.75f, 1.2f, 1.95f}, {23, 1.0f, 1.75f, 1.2f, 1.95f},
+                                 {2, 0.5f, 4.0f, 1.2f, 4.0f}};
+// 16-bit with the rounding residual: 256^3 460 / 283
+constexpr TileCost COST_H16R[] = {{23, 1.2f, 2.1f, 1.7f, 2.4f}, {24, 1.2f, 2.1f, 1.7f, 2.4f},
+                                  {2, 0.55f, 4.5f, 1.7f, 4.5f}};
+// FP64 is bound by the FP64 pipe, which the CTAs of an SM share: 32^3 64 / 22
+constexpr TileCost COST_F64[] = {{6, 0.0f, 49.0f, 0.0f, 49.0f}, {7, 0.0f, 49.0f, 0.0f, 49.0f},
+                                 {2, 0.0f, 54.0f, 0.0f, 54.0f}};
+// D2Q9, FP32 and 16-bit (the floor adds here: co-resident rows overlap):
+// 64^2 4.6 / 2.7, 200^2 4.9 / 3.2, 512^2 7.4 / 5.6, 2000^2 56.5 / 50.5
+constexpr TileCost COST_2D[] = {{4, 0.35f, 0.5f, 0.35f, 0.5f}, {6, 0.35f, 0.6f, 0.35f, 0.6f},
+                                {3, 0.33f, 0.8f, 0.33f, 0.8f}};
+// D2Q9 FP64: 64^2 21.1 / 8.8, 128^2 22.0 / 9.2, 512^2 60 / 54
+constexpr TileCost COST_2D_F64[] = {{1, 2.6f, 25.5f, 2.6f, 25.5f}, {3, 2.6f, 25.5f, 2.6f, 25.5f}};
+
+template <size_t N>
+cudaError_t pick_plan(const TileCost (&cand)[N], int lat, int st, int64_t NX, int64_t NY,
+                      int64_t NZ, FusedPlan *p) {
+  int dev = 0, nsm = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  const double bytes =
+      (double)NX * NY * NZ * 2 * (lat == D3Q19 ? 19 : 9) * (double)storage_bytes(st);
+  const bool in_l2 = bytes < 100e6;
+  const double psi_only = st == ST_F64 ? 0.6 : 2.0;  // the two halo planes, in whole planes
+  double best = 0;
+  bool found = false;
+  for (const TileCost &c : cand) {
+    FusedPlan q;
+    if (fused_make_plan(lat, st, c.tile, NX, NY, NZ, 1, &q) != cudaSuccess) {
+      cudaGetLastError();
+      continue;
+    }
+    int per_sm = 0;
+    if (fused_prepare(lat, st, q, &per_sm) != cudaSuccess || per_sm < 1) {
+      cudaGetLastError();
+      continue;
+    }
+    const int64_t ntiles = (int64_t)q.tiles_x * q.tiles_y;
+    // a ragged last tile takes a plane as long as a full one
+    const double width = (double)std::min<int64_t>(q.bx, lat == D2Q9 ? (NX + 31) / 32 * 32 : NX);
+    const double ns = (in_l2 ? c.ns_l2 : c.ns_hbm) * 1e-3 * width * q.by;
+    const double floor_us = in_l2 ? c.floor_l2 : c.floor_hbm;
+    // every chunk count that can be formed (about 2 sqrt(NZ) of them)
+    for (int64_t zl = NZ; zl >= 1; --zl) {
+      const int64_t n = (NZ + zl - 1) / zl;
+      zl = (NZ + n - 1) / n;
+      if (ntiles * n > INT_MAX) break;
+      const int64_t m = (ntiles * n + nsm - 1) / nsm;  // CTAs of the busiest SM
+      if (q.tile == 25 && lat == D3Q19 && m > per_sm) continue;
+      auto plane = [&](int64_t co) {
+        if (lat == D3Q19) return std::max(floor_us, ns * (double)co);
+        return st == ST_F64 ? std::max(floor_us, 0.6 + ns * (double)co) : floor_us + ns * (double)co;
+      };
+      const double t = ((double)zl + psi_only) * ((double)(m / per_sm) * plane(per_sm) +
+                                                  (m % per_sm ? plane(m % per_sm) : 0.0));
+      const double mem = in_l2 ? 0.0 : bytes * (1.0 + 0.35 / (double)zl) / 6.7e6;
+      // long chunks of a lattice beyond L2 lose the overlap of neighbouring
+      // columns' halo rows (512^3 FP32: 3264 us in 2 chunks, 3160 in 8)
+      const double far = in_l2 ? 1.0 : 1.0 + 0.02 * std::max(0.0, (double)zl / 64 - 1.0);
+      const double cost = (std::max(t, mem) + 0.05 * t) * far;
+      if (!found || cost < best) {
+        best = cost;
+        *p = q;
+        p->zlen = (int)zl;
+        p->nzc = (int)n;
+        p->items = (int)(ntiles * n);
+        found = true;
+      }
+    }
+  }
+  return found ? cudaSuccess : cudaErrorInvalidValue;
+}
+}  // namespace
+
 cudaError_t fused_make_plan(int lat, int st, int tile, int64_t NX, int64_t NY, int64_t NZ,
                             int nzc, FusedPlan *p) {
   int bx, by, ns, xc;
-  if (tile <= 0) tile = 1;
+  if (tile <= 0) {
+    if (lat == D2Q9)
+      return st == ST_F64 ? pick_plan(COST_2D_F64, lat, st, NX, NY, NZ, p)
+                          : pick_plan(COST_2D, lat, st, NX, NY, NZ, p);
+    return st == ST_F64   ? pick_plan(COST_F64, lat, st, NX, NY, NZ, p)
+           : st == ST_F32 ? pick_plan(COST_F32, lat, st, NX, NY, NZ, p)
+           : st == ST_F16R || st == ST_BF16R ? pick_plan(COST_H16R, lat, st, NX, NY, NZ, p)
+                                             : pick_plan(COST_H16, lat, st, NX, NY, NZ, p);
+  }
   if (!fused_tile_shape(lat, st, tile, &bx, &by, &ns, &xc)) return cudaErrorInvalidValue;
   p->tile = tile;
   p->bx = bx;

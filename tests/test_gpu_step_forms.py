@@ -66,3 +66,31 @@ def test_multi_lattice_step_tiles(lbm, lat, ext, nl, storage):
     u = 1.1e-16 if storage == "f64" else 6e-8
     assert rel_err(got, want) < 180 * nl * u
     M.close()
+
+
+@pytest.mark.parametrize("lat,ext", [
+    ("D3Q19", (8, 1, 1)), ("D3Q19", (16, 5, 2)), ("D3Q19", (40, 28, 20)), ("D3Q19", (64, 64, 48)),
+    ("D3Q19", (136, 33, 31)), ("D3Q19", (200, 152, 100)), ("D3Q19", (8, 8, 1500)),
+    ("D2Q9", (8, 1, 1)), ("D2Q9", (64, 64, 1)), ("D2Q9", (200, 131, 1)), ("D2Q9", (1032, 700, 1)),
+    ("D2Q9", (8, 5000, 1))])
+@pytest.mark.parametrize("storage", ["f64", "f32", "f16", "bf16", "f16r", "bf16r"])
+def test_default_plan_gives_the_bits_of_tile_1(lbm, lat, ext, storage):
+    """The plan chosen where the caller names no tile: whatever tile and
+    chunk count it takes (L2-resident and larger lattices, chunks of one
+    plane, one-cell extents), the populations, budgets and residuals are
+    those of tile 1, with an injection site."""
+    nx, ny, nz = ext
+    out = []
+    for tile in (0, 1):
+        L = lbm.Lattice(lat, nx, ny, nz, tau=0.9, G=-5.0, storage=storage.rstrip("r"),
+                        rho_ref=1.8, kernel="fused", tile=tile,
+                        mass_residual=storage.endswith("r"))
+        L.seed_bubbles([[nx / 2, ny / 2, nz // 2, min(nx, max(ny, nz)) / 5]], 1.8, 0.15, 2.0,
+                       1e-3, 5)
+        L.inject([1e-3], [4.5e-3])
+        L.step(7)
+        out.append((L.plan(), L.read("f"), L.read_budgets()))
+        L.close()
+    (plan, f, b), (_, f1, b1) = out
+    assert plan[0] == lbm.KERNEL_FUSED and plan[5] > 0
+    assert (f == f1).all() and (b == b1).all()
