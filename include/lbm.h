@@ -615,20 +615,13 @@ lbm_status lbm_ml_run_until_rupture(lbm_ml_ctx *ctx, const int64_t *line, double
  * back, a time loop that must not stall on the allocator (cudaMalloc and
  * cudaFree can synchronise the device), a program held to a fixed
  * device-memory budget.  It advances FP32 populations f_in -> f_out by one
- * step of the two-pass kernels (no injection).  Layout: Q fields of
- * nx*ny*nz floats, f[i*N + cell], cell = x + nx*(y + ny*z), the
+ * step of the two-pass arithmetic (no injection), one kernel launch.  Layout:
+ * Q fields of nx*ny*nz floats, f[i*N + cell], cell = x + nx*(y + ny*z), the
  * post-streaming form lbm_read(LBM_F) returns, plain values (no offset).
- * The psi field passed between the two kernels lives in a file-scope device
- * array of 2,097,152 floats (8 MB) that every GPU loading the library holds
- * until the process exits; lattices of more cells are rejected with
- * LBM_EINVAL (the product is bounded without overflow).  The first call in
- * each CUDA context (the current one: the device's primary context, or a
- * driver context the caller made current) looks up that array's device
- * address and caches it under the context's process-unique id; make that
- * first call before any stream capture.  Every call uses the same array,
- * which keeps the last call's psi: calls that overlap on the GPU (other
- * streams or threads without ordering) race on it.  f_in and f_out are
- * distinct device buffers owned by the caller; stream may be NULL.
+ * Lattices of more than 2,097,152 cells are rejected with LBM_EINVAL (the
+ * product is bounded without overflow).  Calls share no state: calls on
+ * different buffers may overlap on the GPU.  f_in and f_out are distinct
+ * device buffers owned by the caller; stream may be NULL.
  * Asynchronous; no memory is allocated or freed.  Errors: EINVAL (unknown
  * lattice, extents < 1 or nz != 1 for D2Q9, more than 2,097,152 cells, tau
  * not finite and > 0.5, rho0 not finite and > 0, G not finite, NULL or

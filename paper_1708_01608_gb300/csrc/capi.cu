@@ -78,6 +78,7 @@ struct lbm_ctx {
   FusedPlan plan{};
   FusedMaps tmA{}, tmB{};
   DevBuf psi_scratch;
+  bool march = false;  // LBM_KERNEL_TWO_PASS steps in one launch (step_march.cu)
   // diagnostics
   DevBuf d_err, d_rho, d_p, d_tmp, d_j, d_u, d_labels, d_ncomp, d_part, d_tot, d_site_lab;
   // bubble census and per-point film test
@@ -367,7 +368,10 @@ lbm_status lbm_create(const lbm_config *cfg, lbm_ctx **out) {
       if (cfg->kernel == LBM_KERNEL_FUSED)
         return bail(fail(LBM_EINVAL, "fused kernel: unknown tile, tile too large for this storage, "
                                      "or nx not a multiple of 16 bytes of elements"));
-      c->kernel = LBM_KERNEL_TWO_PASS;  // automatic choice falls back to the two-pass path
+      // automatic choice: the two-pass step, in its one-launch form where
+      // that exists (the residual forms read residuals of neighbours)
+      c->kernel = LBM_KERNEL_TWO_PASS;
+      c->march = !c->resid;
     }
   }
   if (c->kernel == LBM_KERNEL_FUSED) {
@@ -381,7 +385,7 @@ lbm_status lbm_create(const lbm_config *cfg, lbm_ctx **out) {
         fused_encode_maps(c->lat, c->st, c->plan, c->fB.p, c->v.NX, c->v.NY, c->v.NZ, c->v.px,
                           &c->tmB) != CUDA_SUCCESS)
       return bail(fail(LBM_ECUDA, "cuTensorMapEncodeTiled failed"));
-  } else {
+  } else if (!c->march) {
     const size_t cs = c->st == LBM_F64 ? 8 : 4;
     if ((st = dalloc(c, c->psi_scratch, (size_t)c->N * cs)) != LBM_OK) return bail(st);
   }
@@ -647,6 +651,8 @@ lbm_status lbm_step(lbm_ctx *c, int64_t nsteps) {
     cudaError_t e;
     if (c->kernel == LBM_KERNEL_FUSED)
       e = fused_launch(c->lat, c->st_step, c->plan, a, c->cur == 0 ? c->tmA : c->tmB, c->s);
+    else if (c->march)
+      e = march_launch(c->lat, c->st_step, a, c->s);
     else
       e = twopass_launch(c->lat, c->st_step, a, c->psi_scratch.p, c->s);
     if (e == cudaSuccess && spread)

@@ -137,6 +137,10 @@ int fused_x2_smem_bf16(int lat, int tile);
 
 // two-pass path: psi field pass, then collide/stream (+ injection kernel)
 cudaError_t twopass_launch(int lat, int st, const StepArgs &a, void *psi_scratch, cudaStream_t s);
+// injection of the two-pass step: deposits into the populations pushed to fout
+cudaError_t twopass_inject(int lat, int st, const StepArgs &a, cudaStream_t s);
+// the two-pass step without the residual forms as one launch (step_march.cu)
+cudaError_t march_launch(int lat, int st, const StepArgs &a, cudaStream_t s);
 
 // ---- diagnostics / state kernels (diag.cu) --------------------------------
 // n / d for every 32-bit n with one multiply-high and two shifts: division

@@ -3,9 +3,10 @@
 // psi of the neighbours from that field, collides and pushes f*_i to x + c_i.  The blowing-agent
 // injection runs as a third, one-thread-per-site kernel.  This path moves
 // 3*Q*S + 2*sizeof(psi) bytes per update instead of the fused kernel's
-// 2*Q*S; it is kept as a simple, independently written comparison path.
-#include <cmath>
-#include <mutex>
+// 2*Q*S; it is kept as a simple, independently written comparison path and
+// steps the residual forms on rows that are no multiple of 16 bytes.
+#include <algorithm>
+#include <type_traits>
 
 #include "internal.h"
 #include "lattice.cuh"
@@ -210,178 +211,43 @@ __global__ void tp_inject_kernel(const StepArgs a) {
   }
 }
 
-template <int LAT, int ST>
-static cudaError_t tp_launch_t(const StepArgs &a, void *psi, cudaStream_t s) {
-  using C = typename Storage<ST>::C;
-  const int64_t N = a.NX * a.NY * a.NZ;
-  const int threads = 256;
-  const int blocks = (int)((N + threads - 1) / threads < 1048576 ? (N + threads - 1) / threads
-                                                                  : 1048576);
-  tp_psi_kernel<LAT, ST><<<blocks, threads, 0, s>>>(a, static_cast<C *>(psi));
-  tp_collide_kernel<LAT, ST><<<blocks, threads, 0, s>>>(a, static_cast<const C *>(psi));
-  if (a.nsites > 0) tp_inject_kernel<LAT, ST><<<(a.ngroups + 127) / 128, 128, 0, s>>>(a);
-  return cudaGetLastError();
+// f(integral_constant lattice, integral_constant storage) of the runtime pair
+template <class F>
+static cudaError_t tp_dispatch(int lat, int st, F f) {
+  auto with = [&](auto l) {
+    switch (st) {
+      case ST_F64: return f(l, std::integral_constant<int, ST_F64>{});
+      case ST_F32: return f(l, std::integral_constant<int, ST_F32>{});
+      case ST_F16: return f(l, std::integral_constant<int, ST_F16>{});
+      case ST_F16R: return f(l, std::integral_constant<int, ST_F16R>{});
+      case ST_BF16R: return f(l, std::integral_constant<int, ST_BF16R>{});
+      default: return f(l, std::integral_constant<int, ST_BF16>{});
+    }
+  };
+  return lat == D3Q19 ? with(std::integral_constant<int, D3Q19>{})
+                      : with(std::integral_constant<int, D2Q9>{});
+}
+
+cudaError_t twopass_inject(int lat, int st, const StepArgs &a, cudaStream_t s) {
+  return tp_dispatch(lat, st, [&](auto l, auto t) {
+    tp_inject_kernel<decltype(l)::value, decltype(t)::value>
+        <<<(a.ngroups + 127) / 128, 128, 0, s>>>(a);
+    return cudaGetLastError();
+  });
 }
 
 cudaError_t twopass_launch(int lat, int st, const StepArgs &a, void *psi, cudaStream_t s) {
-  if (lat == D3Q19) {
-    switch (st) {
-      case ST_F64: return tp_launch_t<D3Q19, ST_F64>(a, psi, s);
-      case ST_F32: return tp_launch_t<D3Q19, ST_F32>(a, psi, s);
-      case ST_F16: return tp_launch_t<D3Q19, ST_F16>(a, psi, s);
-      case ST_F16R: return tp_launch_t<D3Q19, ST_F16R>(a, psi, s);
-      case ST_BF16R: return tp_launch_t<D3Q19, ST_BF16R>(a, psi, s);
-      default: return tp_launch_t<D3Q19, ST_BF16>(a, psi, s);
-    }
-  }
-  switch (st) {
-    case ST_F64: return tp_launch_t<D2Q9, ST_F64>(a, psi, s);
-    case ST_F32: return tp_launch_t<D2Q9, ST_F32>(a, psi, s);
-    case ST_F16: return tp_launch_t<D2Q9, ST_F16>(a, psi, s);
-    case ST_F16R: return tp_launch_t<D2Q9, ST_F16R>(a, psi, s);
-    case ST_BF16R: return tp_launch_t<D2Q9, ST_BF16R>(a, psi, s);
-    default: return tp_launch_t<D2Q9, ST_BF16>(a, psi, s);
-  }
+  const cudaError_t e = tp_dispatch(lat, st, [&](auto l, auto t) {
+    constexpr int LAT = decltype(l)::value, ST = decltype(t)::value;
+    using C = typename Storage<ST>::C;
+    const int64_t N = a.NX * a.NY * a.NZ;
+    const int threads = 256;
+    const int blocks = (int)std::min<int64_t>((N + threads - 1) / threads, 1048576);
+    tp_psi_kernel<LAT, ST><<<blocks, threads, 0, s>>>(a, static_cast<C *>(psi));
+    tp_collide_kernel<LAT, ST><<<blocks, threads, 0, s>>>(a, static_cast<const C *>(psi));
+    return cudaGetLastError();
+  });
+  return e == cudaSuccess && a.nsites > 0 ? twopass_inject(lat, st, a, s) : e;
 }
 
 }  // namespace sclbm
-
-// ---- allocation-free time step ---------------------------------------------
-// Some callers cannot call cudaMalloc: a host framework that owns the whole
-// device-memory pool and forbids allocations behind its back, a time loop
-// that must not stall on the allocator (cudaMalloc and cudaFree can
-// synchronise the device), or a program held to a fixed memory budget.  The
-// two-pass step needs a psi field between its two kernels; this entry point
-// keeps that field in a file-scope device array of fixed size, so it
-// allocates nothing.  In host code the array's name is only a host-side
-// stand-in: its device address is looked up with cudaGetSymbolAddress, once
-// per CUDA context (keyed by the context's process-unique id, so a second
-// context on the same device, or the new primary context after
-// cudaDeviceReset, gets its own look-up).
-namespace sclbm {
-namespace {
-
-constexpr int64_t kStaticPsiCells = 2097152;  // 8 MB of FP32: up to 128^3 cells
-constexpr int kMaxContexts = 64;
-
-static __device__ __align__(256) float g_static_psi[kStaticPsiCells];
-
-typedef CUresult (*CtxGetCurrentFn)(CUcontext *);
-typedef CUresult (*CtxGetIdFn)(CUcontext, unsigned long long *);
-
-std::mutex g_static_mu;
-struct StaticEntry {
-  unsigned long long ctx_id;
-  float *psi;
-};
-StaticEntry g_static_cache[kMaxContexts];
-int g_static_n = 0, g_static_next = 0;
-
-// driver functions used to identify the current context (fetched once)
-bool ctx_functions(CtxGetCurrentFn *cur, CtxGetIdFn *id) {
-  static CtxGetCurrentFn f_cur = nullptr;
-  static CtxGetIdFn f_id = nullptr;
-  if (!f_cur || !f_id) {
-    void *p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuCtxGetCurrent", &p, 12000, cudaEnableDefault, &q) ==
-            cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      f_cur = reinterpret_cast<CtxGetCurrentFn>(p);
-    p = nullptr;
-    if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &p, 12000, cudaEnableDefault, &q) ==
-            cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      f_id = reinterpret_cast<CtxGetIdFn>(p);
-  }
-  *cur = f_cur;
-  *id = f_id;
-  return f_cur && f_id;
-}
-
-// device address of g_static_psi in the current context (looked up on the
-// first call in each context, then cached)
-cudaError_t static_psi_address(float **out) {
-  CtxGetCurrentFn get_cur;
-  CtxGetIdFn get_id;
-  std::lock_guard<std::mutex> lock(g_static_mu);
-  if (!ctx_functions(&get_cur, &get_id)) return cudaErrorNotSupported;
-  CUcontext ctx = nullptr;
-  if (get_cur(&ctx) != CUDA_SUCCESS) return cudaErrorDeviceUninitialized;
-  if (!ctx) {
-    // no context is current yet: cudaSetDevice makes the current device's
-    // primary context current (it allocates nothing)
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaSetDevice(dev);
-    if (e != cudaSuccess) return e;
-    if (get_cur(&ctx) != CUDA_SUCCESS || !ctx) return cudaErrorDeviceUninitialized;
-  }
-  unsigned long long id = 0;
-  if (get_id(ctx, &id) != CUDA_SUCCESS) return cudaErrorDeviceUninitialized;
-  for (int k = 0; k < g_static_n; ++k)
-    if (g_static_cache[k].ctx_id == id) {
-      *out = g_static_cache[k].psi;
-      return cudaSuccess;
-    }
-  void *p = nullptr;
-  const cudaError_t e = cudaGetSymbolAddress(&p, g_static_psi);
-  if (e != cudaSuccess) return e;
-  // a full table reuses its oldest entry: a context evicted that way is
-  // looked up again on its next call
-  const int slot = g_static_n < kMaxContexts ? g_static_n++ : g_static_next;
-  if (g_static_n == kMaxContexts) g_static_next = (slot + 1) % kMaxContexts;
-  g_static_cache[slot] = StaticEntry{id, static_cast<float *>(p)};
-  *out = static_cast<float *>(p);
-  return cudaSuccess;
-}
-
-}  // namespace
-}  // namespace sclbm
-
-extern "C" lbm_status lbm_step_static_f32(int32_t lattice, int64_t nx, int64_t ny, int64_t nz,
-                                          double tau, double G, double rho0, const float *f_in,
-                                          float *f_out, void *stream) {
-  using namespace sclbm;
-  if (lattice != LBM_D2Q9 && lattice != LBM_D3Q19)
-    return set_error(LBM_EINVAL, "lbm_step_static_f32: unknown lattice");
-  if (nx < 1 || ny < 1 || nz < 1 || (lattice == LBM_D2Q9 && nz != 1))
-    return set_error(LBM_EINVAL, "lbm_step_static_f32: extents must be >= 1 (nz = 1 for D2Q9)");
-  // nx * ny * nz <= cap, tested by division so that no product can overflow
-  if (nx > kStaticPsiCells || ny > kStaticPsiCells / nx || nz > kStaticPsiCells / (nx * ny))
-    return set_error(LBM_EINVAL,
-                     "lbm_step_static_f32: more than 2097152 cells, the size of the static "
-                     "scratch array (use lbm_create/lbm_step for larger lattices)");
-  if (!(tau > 0.5) || !std::isfinite(tau) || !(rho0 > 0) || !std::isfinite(rho0) ||
-      !std::isfinite(G))
-    return set_error(LBM_EINVAL,
-                     "lbm_step_static_f32: tau must be finite and > 0.5, rho0 finite and > 0, "
-                     "G finite");
-  if (!f_in || !f_out || static_cast<const void *>(f_in) == static_cast<const void *>(f_out))
-    return set_error(LBM_EINVAL, "lbm_step_static_f32: f_in and f_out must be distinct buffers");
-  float *psi = nullptr;
-  cudaError_t e = static_psi_address(&psi);
-  if (e != cudaSuccess) {
-    cudaGetLastError();
-    return set_error(LBM_ECUDA, cudaGetErrorString(e));
-  }
-  StepArgs a{};
-  a.fin = f_in;
-  a.fout = f_out;
-  a.NX = nx;
-  a.NY = lattice == LBM_D2Q9 ? 1 : ny;  // D2Q9 runs on the view (nx, 1, ny)
-  a.NZ = lattice == LBM_D2Q9 ? ny : nz;
-  a.px = nx;
-  a.tau = tau;
-  a.G = G;
-  a.rho0 = rho0;
-  a.rho_ref = 0.0;  // plain f_i, no offset
-  a.nsites = 0;
-  const cudaStream_t s = static_cast<cudaStream_t>(stream);
-  e = lattice == LBM_D2Q9 ? tp_launch_t<D2Q9, ST_F32>(a, psi, s) : tp_launch_t<D3Q19, ST_F32>(a, psi, s);
-  if (e != cudaSuccess) {
-    cudaGetLastError();
-    return set_error(LBM_ECUDA, cudaGetErrorString(e));
-  }
-  return LBM_OK;
-}

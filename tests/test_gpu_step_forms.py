@@ -94,3 +94,72 @@ def test_default_plan_gives_the_bits_of_tile_1(lbm, lat, ext, storage):
     (plan, f, b), (_, f1, b1) = out
     assert plan[0] == lbm.KERNEL_FUSED and plan[5] > 0
     assert (f == f1).all() and (b == b1).all()
+
+
+ROWS = [("D3Q19", (1, 1, 1)), ("D3Q19", (1, 9, 4)), ("D3Q19", (29, 6, 3)), ("D3Q19", (30, 7, 2)),
+        ("D3Q19", (31, 5, 1)), ("D3Q19", (61, 23, 70)), ("D3Q19", (33, 1, 5)), ("D2Q9", (1, 1, 1)),
+        ("D2Q9", (125, 9, 1)), ("D2Q9", (126, 8, 1)), ("D2Q9", (127, 1500, 1)), ("D2Q9", (255, 2, 1))]
+
+
+@pytest.mark.parametrize("lat,ext", ROWS)
+@pytest.mark.parametrize("storage", ["f32", "f16", "bf16"])
+def test_one_launch_step_gives_the_bits_of_the_two_pass_step(lbm, lat, ext, storage):
+    """Rows that are no multiple of 16 bytes, at the edges of the march's
+    tiles (30 x 6 and 126 cells) and chunks: the step an automatic choice
+    takes there has the populations and budgets of the two-pass kernels, with
+    two injection sites in one cell and a neighbouring one."""
+    nx, ny, nz = ext
+    out = []
+    for kernel in ("auto", "two_pass"):
+        L = lbm.Lattice(lat, nx, ny, nz, tau=0.9, G=-5.0, storage=storage, rho_ref=1.8,
+                        kernel=kernel)
+        x, y, z = nx // 2, ny // 2, nz // 2
+        L.seed_bubbles([[x, y, z, nx / 5], [x, y, z, 1.0], [(x + 1) % nx, y, z, 1.0]], 1.8, 0.15,
+                       2.0, 1e-3, 5)
+        L.inject([1e-3, 2e-3, 3e-3], [4.5e-3, 9e-3, 1.0])
+        L.step(7)
+        out.append((L.plan()[0], L.read("f"), L.read_budgets()))
+        L.close()
+    (kind, f, b), (kind1, f1, b1) = out
+    assert kind == kind1 == lbm.KERNEL_TWO_PASS
+    assert (f == f1).all() and (b == b1).all()
+
+
+@pytest.mark.parametrize("lat,ext", ROWS)
+def test_one_launch_step_fp64(lbm, lat, ext):
+    """The FP64 form on odd rows: one step, 40 roundings of at most rho per
+    population as above (2e-14 of the largest population)."""
+    nx, ny, nz = ext
+    q = 19 if lat == "D3Q19" else 9
+    _, w = O.velocities(LAT[lat])
+    rng = np.random.default_rng(nx + ny)
+    f0 = (w[:, None, None, None] * rng.uniform(0.1, 2.0, size=(1, nz, ny, nx))
+          * rng.uniform(0.9, 1.1, size=(q, nz, ny, nx)))
+    L = lbm.Lattice(lat, nx, ny, nz, tau=0.8, G=-5.0, storage="f64")
+    L.write_f(f0)
+    L.step(1)
+    assert rel_err(L.read("f"), O.run(LAT[lat], f0, 1, 0.8, -5.0)) < 2e-14
+    L.close()
+
+
+@pytest.mark.parametrize("lat,ext", ROWS + [("D3Q19", (32, 12, 3)), ("D2Q9", (128, 4, 1))])
+def test_static_step_gives_the_bits_of_the_two_pass_step(lbm, lat, ext):
+    import torch
+    nx, ny, nz = ext
+    q = 19 if lat == "D3Q19" else 9
+    _, w = O.velocities(LAT[lat])
+    rng = np.random.default_rng(nx * ny)
+    f0 = (w[:, None, None, None] * rng.uniform(0.1, 2.0, size=(1, nz, ny, nx))
+          * rng.uniform(0.9, 1.1, size=(q, nz, ny, nx))).astype(np.float32)
+    L = lbm.Lattice(lat, nx, ny, nz, tau=0.8, G=-5.0, storage="f32", kernel="two_pass",
+                    rho_ref=0.0)
+    L.write_f(f0.astype(np.float64))
+    L.step(4)
+    a = torch.from_numpy(f0).cuda()
+    b = torch.empty_like(a)
+    for _ in range(4):
+        lbm.step_static_f32(lat, nx, ny, nz, 0.8, -5.0, 1.0, a.data_ptr(), b.data_ptr(),
+                            torch.cuda.current_stream().cuda_stream)
+        a, b = b, a
+    assert (a.cpu().numpy().astype(np.float64) == L.read("f").reshape(f0.shape)).all()
+    L.close()
