@@ -13,8 +13,11 @@
 // into a four-plane psi ring in shared memory, the inner ones collide the
 // plane before it.  Rings cost loads (L2 hits) in place of a divergent halo
 // pass.  The next plane's populations are in flight, in registers, over the
-// barrier and the collision; the colliding plane's are read a second time,
-// from L1, since a third set of registers would halve the CTAs of an SM.
+// barrier and the collision; the colliding plane's wait in shared memory, each
+// thread in its own slots (read a second time instead they came from L2, 2 %
+// of them from L1: 49.0 us at 127x101x90 against 43.5; in a third set of
+// registers, with two CTAs per SM, 44.0).  FP64, which the pipe bounds, reads
+// them twice.
 //
 // FP32 arithmetic repeats the two-pass kernels rounding for rounding and
 // gives their bits (the state after a step, and so every label and census
@@ -24,7 +27,7 @@
 // us per step, two-pass / this: 201x150x99 FP32 168 / 121, FP16 164 / 97;
 // 33x35x31 FP32 10.3 / 4.9; 93^3 FP64 772 / 451; D2Q9 201^2 FP32 10.3 / 3.0,
 // 1401x1203 68 / 25, 129^2 FP64 27 / 11; the allocation-free step at
-// 127x101x90 54 / 50.  Blocks of 32 x 8 threads, three per SM, against 32 x
+// 127x101x90 54 / 43.5.  Blocks of 32 x 8 threads, three per SM, against 32 x
 // 12, two per SM (124 and 105 at 201x150x99) and 32 x 24 (144 and 118);
 // without the plane in flight 129 and 112.
 #include <algorithm>
@@ -58,6 +61,7 @@ __global__ void __launch_bounds__(TX *TY, MINB)
   static_assert(BX > 0 && BY > 0 && (HY || TY == 1), "a cell inside the halo ring");
   static_assert(!S::RESID, "psi reads neighbours' residuals, which the collision rewrites");
   __shared__ C ring[4][TY][TX];
+  __shared__ T held[F64 ? 1 : 2][Q][F64 ? 1 : TX * TY];  // planes P and P - 1
 
   const int NX = (int)a.NX, NY = (int)a.NY, NZ = (int)a.NZ;
   const int tx = threadIdx.x % TX, ty = threadIdx.x / TX;
@@ -111,6 +115,8 @@ __global__ void __launch_bounds__(TX *TY, MINB)
         for (int i = 0; i < Q; ++i) r += S::load(next[i]);
         r1 = r;
         ring[k & 3][ty][tx] = psi_of(r + rho_ref, rho0, inv_rho0);
+#pragma unroll
+        for (int i = 0; i < Q; ++i) held[k & 1][i][threadIdx.x] = next[i];
         if (k + 1 < npl) load_plane(P + 1);
       }
     }
@@ -121,7 +127,6 @@ __global__ void __launch_bounds__(TX *TY, MINB)
     const int Pc = P - 1;
     const int oz[3] = {(Pc == 0 ? NZ - 1 : Pc - 1) * plane, Pc * plane,
                        (Pc + 1 >= NZ ? 0 : Pc + 1) * plane};
-    const T *own = fin + (oz[1] + oy[1] + x);
     auto psi_at = [&](int i) -> C {
       return ring[(k - 1 + L::cz(i)) & 3][ty + L::cy(i)][tx + L::cx(i)];
     };
@@ -130,6 +135,7 @@ __global__ void __launch_bounds__(TX *TY, MINB)
              (oz[L::cz(i) + 1] + oy[L::cy(i) + 1] + ox[L::cx(i) + 1]);
     };
     if constexpr (F64) {
+      const T *own = fin + (oz[1] + oy[1] + x);
       T f[Q];
 #pragma unroll
       for (int i = 0; i < Q; ++i) f[i] = own[i * pop];
@@ -140,7 +146,7 @@ __global__ void __launch_bounds__(TX *TY, MINB)
     } else {
       C g[Q];
 #pragma unroll
-      for (int i = 0; i < Q; ++i) g[i] = S::load(own[i * pop]);
+      for (int i = 0; i < Q; ++i) g[i] = S::load(held[(k - 1) & 1][i][threadIdx.x]);
       // every rounding written out, as the two-pass kernels have it; the
       // relaxation of opposite velocities runs as paired instructions
       C sx = 0, sy = 0, sz = 0, jx = 0, jy = 0, jz = 0;
