@@ -78,7 +78,9 @@ struct lbm_ctx {
   FusedPlan plan{};
   FusedMaps tmA{}, tmB{};
   DevBuf psi_scratch;
-  bool march = false;  // LBM_KERNEL_TWO_PASS steps in one launch (step_march.cu)
+  // LBM_KERNEL_TWO_PASS steps in one launch: on plain loads (step_march.cu),
+  // or with plan (tmA, tmB) through the x-pair kernel's ROWS form
+  bool march = false, rows = false;
   // diagnostics
   DevBuf d_err, d_rho, d_p, d_tmp, d_j, d_u, d_labels, d_ncomp, d_part, d_tot, d_site_lab;
   // bubble census and per-point film test
@@ -107,6 +109,13 @@ struct lbm_ctx {
 };
 
 namespace {
+
+// Rows that are no multiple of 16 bytes: from this many cells on the x-pair
+// kernel's form for them, below it the march on plain loads, whose smaller
+// tiles spread a small lattice over more SMs.  us per step, march / x-pair
+// form: FP32 49^3 7.7 / 10.2, 65^3 13.8 / 18.6, 81^3 22.2 / 24.7, 99^3 43.0 /
+// 35.3, 127^3 80 / 58; FP16 65^3 13.7 / 14.9, 81^3 22.1 / 20.4, 127^3 68 / 44.
+constexpr int64_t kRowsMinCells = 600000;
 
 void hfree(PinBuf &b) {
   if (b.p) cudaFreeHost(b.p);
@@ -368,13 +377,20 @@ lbm_status lbm_create(const lbm_config *cfg, lbm_ctx **out) {
       if (cfg->kernel == LBM_KERNEL_FUSED)
         return bail(fail(LBM_EINVAL, "fused kernel: unknown tile, tile too large for this storage, "
                                      "or nx not a multiple of 16 bytes of elements"));
-      // automatic choice: the two-pass step, in its one-launch form where
-      // that exists (the residual forms read residuals of neighbours)
+      // automatic choice: the two-pass step, in one of its one-launch forms
+      // where they exist (the residual forms read residuals of neighbours):
+      // the x-pair kernel on padded rows, else the march on plain loads
       c->kernel = LBM_KERNEL_TWO_PASS;
-      c->march = !c->resid;
+      if (!c->resid && c->lat == D3Q19 && c->st != LBM_F64 && cfg->tile <= 0 &&
+          c->N >= kRowsMinCells) {
+        c->rows = fused_make_plan(c->lat, c->st_step, 0, c->v.NX, c->v.NY, c->v.NZ, 0, &c->plan,
+                                  true) == cudaSuccess;
+        cudaGetLastError();
+      }
+      c->march = !c->resid && !c->rows;
     }
   }
-  if (c->kernel == LBM_KERNEL_FUSED) {
+  if (c->kernel == LBM_KERNEL_FUSED || c->rows) {
     cudaError_t e = fused_prepare(c->lat, c->st_step, c->plan);
     if (e != cudaSuccess) {
       cudaGetLastError();
@@ -651,7 +667,12 @@ lbm_status lbm_step(lbm_ctx *c, int64_t nsteps) {
     cudaError_t e;
     if (c->kernel == LBM_KERNEL_FUSED)
       e = fused_launch(c->lat, c->st_step, c->plan, a, c->cur == 0 ? c->tmA : c->tmB, c->s);
-    else if (c->march)
+    else if (c->rows) {
+      StepArgs b = a;  // the deposits are a kernel of their own
+      b.nsites = 0;
+      e = fused_launch(c->lat, c->st_step, c->plan, b, c->cur == 0 ? c->tmA : c->tmB, c->s);
+      if (e == cudaSuccess && a.nsites > 0) e = twopass_inject(c->lat, c->st_step, a, c->s);
+    } else if (c->march)
       e = march_launch(c->lat, c->st_step, a, c->s);
     else
       e = twopass_launch(c->lat, c->st_step, a, c->psi_scratch.p, c->s);
@@ -1317,8 +1338,7 @@ lbm_status lbm_diagnostic_interval(lbm_ctx *c, int32_t h_max, double eps_arm, in
       CK(cudaMemcpyAsync(mail + 8, c->d_tot.p, 32, cudaMemcpyDeviceToHost, c->s));
       CK(cudaMemcpyAsync(mail + 40, c->d_film_counts.p, 40, cudaMemcpyDeviceToHost, c->s));
       if (labels)
-        CK(cudaMemcpyAsync(labels, c->d_labels.p, sizeof(int32_t) * c->N, cudaMemcpyDeviceToHost,
-                           c->s));
+        CK(cudaMemcpyAsync(labels, c->d_labels.p, sizeof(int32_t) * c->N, cudaMemcpyDeviceToHost, c->s));
       if (rec_bytes)
         CK(cudaMemcpyAsync(mail + 80 + block, c->d_film_rec.p, rec_bytes, cudaMemcpyDeviceToHost,
                            c->s));

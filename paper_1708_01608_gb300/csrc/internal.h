@@ -77,6 +77,7 @@ struct FusedPlan {
   int smem;      // dynamic shared memory bytes
   int hx;        // halo columns per box (16 bytes of elements)
   int xc;        // cells per thread along x: 1, or 2 for the x-pair kernel
+  bool rows = false;  // the x-pair kernel's form for rows that are no multiple of 16 bytes
 };
 
 // Tile shapes: returns false when the id is unknown for the lattice and
@@ -87,9 +88,9 @@ bool fused_tile_shape(int lat, int st, int tile, int *bx, int *by, int *nstage,
 // with the fewest staged planes per resident CTA slot when the CTAs run in
 // waves of SMs x CTAs per SM; -1: as many as fill those slots once.  Returns
 // cudaErrorInvalidValue when the tile does not fit or nx is not a multiple
-// of the 16-byte halo width.
+// of the 16-byte halo width (unless rows asks for the form that takes any).
 cudaError_t fused_make_plan(int lat, int st, int tile, int64_t NX, int64_t NY, int64_t NZ,
-                            int nzc, FusedPlan *plan);
+                            int nzc, FusedPlan *plan, bool rows = false);
 // Encode the TMA descriptors of one population lattice for a plan.
 CUresult fused_encode_maps(int lat, int st, const FusedPlan &plan, const void *base,
                            int64_t NX, int64_t NY, int64_t NZ, int64_t px, FusedMaps *tm);

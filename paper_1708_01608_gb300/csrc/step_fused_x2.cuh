@@ -22,6 +22,17 @@
 // P - 1 (holding two planes of float pairs would cost 38 registers): its
 // stage is free one iteration after it was consumed, and NS - 1 planes are
 // in flight ahead of the plane being summed.
+//
+// ROWS is the form for rows that are no multiple of 16 bytes (the pitch is):
+// the periodic halo column NX - 1 sits inside its 16-byte box instead of at
+// its end, and with an odd NX the last pair's cell b is padding.  b's pushes
+// then go to the padding column or nowhere else, so no store is predicated.
+// Its arithmetic is that of the two-pass kernels, rounding for rounding
+// (plain sums in velocity order, IEEE division): the step of such a lattice
+// has their bits.  Against the march on plain loads (step_march.cu) the
+// staging takes a population through L2 once and a thread does two cells: us
+// per step at 201x150x99 FP32 121 / 91, FP16 97 / 71, at 333x301x250 FP16 790 /
+// 481 (HBM at its copy rate: 67, 33 and 281).
 #pragma once
 
 #include "step_fused.cuh"
@@ -33,6 +44,11 @@ __device__ __forceinline__ float2 f2(float v) { return make_float2(v, v); }
 __device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
 __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+// a b, rounded, where a sum follows: a paired multiply and add written apart
+// may become one FMA, which the scalar intrinsics exclude
+__device__ __forceinline__ float2 mulr2(float2 a, float2 b) {
+  return make_float2(__fmul_rn(a.x, b.x), __fmul_rn(a.y, b.y));
+}
 // a - b, rounded once (b * -1 is exact)
 __device__ __forceinline__ float2 sub2(float2 a, float2 b) {
   return __ffma2_rn(b, make_float2(-1.0f, -1.0f), a);
@@ -188,6 +204,15 @@ __device__ __forceinline__ float2 sum_q_w2(Ld ld) {
   return __fadd2_rn(make_float2(ax, ay), make_float2(bx, by));
 }
 
+// the plain sum in velocity order, from 0 (the two-pass kernels')
+template <int Q, class V, class Ld>
+__device__ __forceinline__ V sum_seq(Ld ld) {
+  V a{};
+#pragma unroll
+  for (int i = 0; i < Q; ++i) a = addv(a, ld(i));
+  return a;
+}
+
 template <int LAT, int ST, int BX_, int BY_, int NS_>
 struct FusedK2 {
   using B = FusedK<LAT, ST, BX_, BY_, NS_>;
@@ -213,7 +238,7 @@ struct FusedK2 {
 
 // OM16: 1 - omega is exactly a value of the 16-bit storage type, so the
 // relaxation's (1 - omega) g_i takes the stored g_i unconverted (fma_w)
-template <int LAT, int ST, int BX, int BY, int NS, bool OM16 = false, class OutPop>
+template <int LAT, int ST, int BX, int BY, int NS, bool OM16 = false, bool ROWS = false, class OutPop>
 __device__ __forceinline__ bool fused_march_x2(const MarchArgs &m, OutPop out_pop, uint32_t &kb) {
   using K = FusedK2<LAT, ST, BX, BY, NS>;
   using B = typename K::B;
@@ -228,6 +253,7 @@ __device__ __forceinline__ bool fused_march_x2(const MarchArgs &m, OutPop out_po
   // 16-bit residual forms: each cell's rounding residual of the last step
   // joins its mass R, and the new one is what this step's stores round off
   constexpr bool RESID = S1::RESID;
+  static_assert(!(ROWS && (RESID || OM16)), "ROWS: plain storage, two-pass arithmetic");
   // 16-bit storage keeps a staged plane in registers as packed pairs (19
   // registers): read from its stage once, for psi, it is collided one
   // iteration later, and the stage is refilled right after the psi phase,
@@ -247,11 +273,13 @@ __device__ __forceinline__ bool fused_march_x2(const MarchArgs &m, OutPop out_po
   const int tx = 2 * tp;  // tile column of cell a; cell b is tx + 1
   const int NX = m.NX, NY = m.NY, NZ = m.NZ;
   const int x0 = m.x0, y0 = m.y0, zs = m.zs, ze = m.ze;
-  const int BXe = min(BX, NX - x0), BYe = min(BY, NY - y0);  // BXe is even
+  const int BXe = min(BX, NX - x0), BYe = min(BY, NY - y0);  // BXe is even but for ROWS
   if (zs >= ze) return true;
   const int NPL = ze - zs + 2;  // staged planes zs-1 .. ze
   const bool active = tx < BXe && ty < BYe;
-  const int xl = x0 == 0 ? NX - HX : x0 - HX;
+  const int xl = x0 > 0 ? x0 - HX : (ROWS ? (NX - 1) / HX * HX : NX - HX);
+  const int el = ROWS && x0 == 0 ? (NX - 1) % HX : HX - 1;  // the halo column in its box
+  const bool has_b = !ROWS || tx + 1 < BXe;
   const int xr = x0 + BXe == NX ? 0 : x0 + BXe;
   const int yt = y0 == 0 ? NY - 1 : y0 - 1;
   const int yb = y0 + BYe == NY ? 0 : y0 + BYe;
@@ -306,7 +334,11 @@ __device__ __forceinline__ bool fused_march_x2(const MarchArgs &m, OutPop out_po
   // only a's -x and b's +x destinations can wrap.
   const int x = x0 + tx, y = y0 + ty;
   const int32_t dam = (x == 0 ? NX - 1 : x - 1) - x;  // a, cx = -1: -1 or NX - 1
-  const int32_t dbp = (x + 2 >= NX ? 0 : x + 2) - x;  // b, cx = +1: 2 or -x
+  const int32_t dbp = ROWS && !has_b ? 1 : (x + 2 >= NX ? 0 : x + 2) - x;  // b, cx = +1: 2 or -x
+  // ROWS: a's +x push wraps where it is the last cell; a missing b pushes to
+  // its own place, the padding column x + 1
+  const int32_t dap = ROWS && !has_b ? (x + 1 >= NX ? -x : 1) : 1;
+  const int32_t dbm = ROWS && !has_b ? 1 : 0;
   const int ym = y == 0 ? NY - 1 : y - 1, yp = y + 1 >= NY ? 0 : y + 1;
   const int32_t oy[3] = {(int32_t)(ym * m.px), (int32_t)(y * m.px), (int32_t)(yp * m.px)};
 
@@ -314,17 +346,18 @@ __device__ __forceinline__ bool fused_march_x2(const MarchArgs &m, OutPop out_po
   // row, or one cell of the corners and side columns.  h_off: byte offset of
   // its population 0 in a stage; h_pstride: elements between populations;
   // h_j: its ring index (column of cell a).
-  const int nunits = HY ? BXe + 4 + 2 * BYe : 2;
+  const int nunits = HY ? (ROWS ? (BXe + 1) / 2 * 2 : BXe) + 4 + 2 * BYe : 2;
   int h_off = 0, h_pstride = 0, h_j = 0;
-  bool h_pair = false;
+  bool h_pair = false, h_b = true;  // h_b: the pair's second cell is in the tile
   if (tid < nunits) {
     int dx, dy;
     if (HY) {
-      const int np = BXe / 2;
+      const int np = ROWS ? (BXe + 1) / 2 : BXe / 2;
       if (tid < 2 * np) {
         h_pair = true;
         dy = tid < np ? -1 : BYe;
         dx = 2 * (tid < np ? tid : tid - np);
+        h_b = !ROWS || dx + 1 < BXe;
       } else if (tid < 2 * np + 4) {
         const int h = tid - 2 * np;
         dx = (h & 1) ? BXe : -1;
@@ -343,7 +376,7 @@ __device__ __forceinline__ bool fused_march_x2(const MarchArgs &m, OutPop out_po
     int off, e;
     if (cyr == 1) {  // side column (never the interior)
       off = cxr == 0 ? B::OFF_L : B::OFF_R;
-      e = dy * HX + (cxr == 0 ? HX - 1 : 0);
+      e = dy * HX + (cxr == 0 ? el : 0);
       h_pstride = BY * HX;
     } else if (cxr == 1) {  // top or bottom row
       off = cyr == 0 ? B::OFF_T : B::OFF_B;
@@ -351,7 +384,7 @@ __device__ __forceinline__ bool fused_march_x2(const MarchArgs &m, OutPop out_po
       h_pstride = BX;
     } else {
       off = cyr == 0 ? (cxr == 0 ? B::OFF_TL : B::OFF_TR) : (cxr == 0 ? B::OFF_BL : B::OFF_BR);
-      e = cxr == 0 ? HX - 1 : 0;
+      e = cxr == 0 ? el : 0;
       h_pstride = HX;
     }
     h_off = off + e * (int)sizeof(T);
@@ -392,14 +425,17 @@ __device__ __forceinline__ bool fused_march_x2(const MarchArgs &m, OutPop out_po
         for (int i = 0; i < Q; ++i) nxt[i] = main2[(i * BY + ty) * TPX + tp];
       }
       float2 r2;
-      if constexpr (sizeof(T) == 2)
+      if constexpr (ROWS)
+        r2 = sum_seq<Q, float2>(
+            [&](int i) { return S2::load(KEEP ? nxt[i] : main2[(i * BY + ty) * TPX + tp]); });
+      else if constexpr (sizeof(T) == 2)
         r2 = sum_q_w2<Q>([&](int i) { return KEEP ? nxt[i] : main2[(i * BY + ty) * TPX + tp]; });
       else
         r2 = sum_q<Q, float2>([&](int i) { return S2::load(main2[(i * BY + ty) * TPX + tp]); });
       const float2 ps = psi_x2(add2(f2(rho_ref), r2), rho0, inv_rho0);
       *reinterpret_cast<float2 *>(rN + c0) = ps;
       rS[c0 - 1] = ps.x;
-      rS[c0] = ps.y;
+      if (has_b) rS[c0] = ps.y;  // else the slot of the halo column
       Rnxt = r2;
     }
     if (tid < nunits) {
@@ -407,18 +443,22 @@ __device__ __forceinline__ bool fused_march_x2(const MarchArgs &m, OutPop out_po
         const T2 *b2 = reinterpret_cast<const T2 *>(st + h_off);
         const int ps2 = h_pstride / 2;
         float2 r2;
-        if constexpr (sizeof(T) == 2)
+        if constexpr (ROWS)
+          r2 = sum_seq<Q, float2>([&](int i) { return S2::load(b2[i * ps2]); });
+        else if constexpr (sizeof(T) == 2)
           r2 = sum_q_w2<Q>([&](int i) { return b2[i * ps2]; });
         else
           r2 = sum_q<Q, float2>([&](int i) { return S2::load(b2[i * ps2]); });
         const float2 ps = psi_x2(add2(f2(rho_ref), r2), rho0, inv_rho0);
         *reinterpret_cast<float2 *>(rN + h_j) = ps;
         rS[h_j - 1] = ps.x;
-        rS[h_j] = ps.y;
+        if (h_b) rS[h_j] = ps.y;
       } else {
         const T *b1 = reinterpret_cast<const T *>(st + h_off);
         float r;
-        if constexpr (sizeof(T) == 2)
+        if constexpr (ROWS)
+          r = sum_seq<Q, float>([&](int i) { return S1::load(b1[i * h_pstride]); });
+        else if constexpr (sizeof(T) == 2)
           r = sum_q_w1<Q>([&](int i) { return b1[i * h_pstride]; });
         else
           r = sum_q<Q, float>([&](int i) { return S1::load(b1[i * h_pstride]); });
@@ -493,11 +533,11 @@ __device__ __forceinline__ bool fused_march_x2(const MarchArgs &m, OutPop out_po
           } else {
             const T qa = S1::store(v.x), qb = S1::store(v.y);
             if constexpr (cx > 0) {
-              p[1] = qa;
+              p[dap] = qa;
               p[dbp] = qb;
             } else {
               p[dam] = qa;
-              p[0] = qb;
+              p[dbm] = qb;
             }
             if constexpr (RESID)
               racc = add2(racc, make_float2(v.x - S1::load(qa), v.y - S1::load(qb)));
@@ -508,6 +548,48 @@ __device__ __forceinline__ bool fused_march_x2(const MarchArgs &m, OutPop out_po
         const int32_t own = oz[1] + oy[1] + x;  // cell a; b is own + 1
         float2 R = Rcur;
         if constexpr (RESID) R = add2(R, *reinterpret_cast<const float2 *>(m.resid + own));
+        if constexpr (ROWS) {
+          // the two-pass kernels' roundings (step_march.cu), two cells each
+          float2 jx = f2(0.0f), jy = jx, jz = jx, sx = jx, sy = jx, sz = jx;
+          static_for<Q>([&](auto ic) {
+            constexpr int i = decltype(ic)::value;
+            if constexpr (i > 0) {
+              constexpr int cx = L::cx(i), cy = L::cy(i), cz = L::cz(i);
+              const float2 wp = mulr2(f2((float)L::w(i)), psi2_at(ic)), g = S2::load(cur[i]);
+              sx = cacc2<cx>(sx, wp);
+              sy = cacc2<cy>(sy, wp);
+              sz = cacc2<cz>(sz, wp);
+              jx = cacc2<cx>(jx, g);
+              jy = cacc2<cy>(jy, g);
+              jz = cacc2<cz>(jz, g);
+            }
+          });
+          const float2 rho = add2(f2(rho_ref), R);
+          const float2 ir = make_float2(__fdiv_rn(1.0f, rho.x), __fdiv_rn(1.0f, rho.y));
+          const float2 tg = mul2(
+              f2(tau), mul2(f2(-G), *reinterpret_cast<const float2 *>(ringN + k0p * RP + c0)));
+          const float2 ux = mulr2(fma2(tg, sx, jx), ir), uy = mulr2(fma2(tg, sy, jy), ir),
+                       uz = mulr2(fma2(tg, sz, jz), ir);
+          const float2 uu = fma2(uz, uz, fma2(ux, ux, mul2(uy, uy)));
+          const float2 Kc = fma2(mul2(f2(-1.5f), rho), uu, R);
+          float2 moved = f2(0.0f);
+          static_assert(L::HAS_Y, "opposite velocities are neighbours in the order of the sum");
+          static_for<L::NP>([&](auto kc) {
+            constexpr int i = L::rep(decltype(kc)::value), o = L::opp(i);
+                        const float2 cu = cdot2<L::cx(i), L::cy(i), L::cz(i)>(ux, uy, uz);
+            const float2 q = mul2(mul2(f2(4.5f), cu), cu);
+            auto relax = [&](float2 e, float2 g) {
+              const float2 t = fma2(f2(-(float)L::w(i)), fma2(rho, e, Kc), g);
+              return fma2(f2(-omega), t, g);
+            };
+            const float2 gi = relax(fma2(f2(3.0f), cu, q), S2::load(cur[i]));
+            const float2 go = relax(fma2(f2(-3.0f), cu, q), S2::load(cur[o]));
+            moved = add2(add2(moved, gi), go);
+            put(std::integral_constant<int, i>{}, gi);
+            put(std::integral_constant<int, o>{}, go);
+          });
+          put(std::integral_constant<int, 0>{}, sub2(R, moved));
+        } else {
         float2 jx = f2(-0.0f), jy = f2(-0.0f), jz = f2(-0.0f);
         float2 sx = f2(-0.0f), sy = f2(-0.0f), sz = f2(-0.0f);
         static_for<L::NP>([&](auto kc) {
@@ -582,6 +664,7 @@ __device__ __forceinline__ bool fused_march_x2(const MarchArgs &m, OutPop out_po
         else
           relax_push(std::false_type{});
         if constexpr (RESID) *reinterpret_cast<float2 *>(m.resid + own) = racc;
+        }
       }
     }
     // ---- plane P is collided in the next iteration
@@ -598,7 +681,7 @@ __device__ __forceinline__ bool fused_march_x2(const MarchArgs &m, OutPop out_po
   return true;
 }
 
-template <int LAT, int ST, int BX, int BY, int NS, bool OM16 = false>
+template <int LAT, int ST, int BX, int BY, int NS, bool OM16 = false, bool ROWS = false>
 __global__ void __launch_bounds__(BX / 2 * BY, BX / 2 * BY <= 256 ? 512 / (BX / 2 * BY) : 1)
     fused_step_kernel_x2(const __grid_constant__ FusedMaps tm, const StepArgs a, const int tiles_x,
                          const int tiles_y, const int zlen) {
@@ -609,7 +692,7 @@ __global__ void __launch_bounds__(BX / 2 * BY, BX / 2 * BY <= 256 ? 512 / (BX / 
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   uint32_t kb = 0;
-  fused_march_x2<LAT, ST, BX, BY, NS, OM16>(
+  fused_march_x2<LAT, ST, BX, BY, NS, OM16, ROWS>(
       m, [&](int i) { return static_cast<T *>(a.out_pop[i]); }, kb);
 }
 
@@ -629,9 +712,28 @@ bool om1_is_16bit(float omega) {
   }
 }
 
+// The tiles that have a ROWS form: those the default plan takes for the
+// storage (D3Q19; D2Q9 rows step through step_march.cu, as fast there: 201^2
+// FP32 3.0 us against 3.2 for this kernel at 200^2)
 template <int LAT, int ST, int BX, int BY, int NS>
-cudaError_t fused_x2_prepare_t(int *blocks_per_sm) {
+constexpr bool HAS_ROWS = LAT == D3Q19 && !Storage<ST>::RESID &&
+                          NS == (sizeof(typename Storage<ST>::T) == 4 ? 3 : 2) &&
+                          ((BX == 64 && BY == 8) || (BX == 128 && BY == 4));
+
+template <int LAT, int ST, int BX, int BY, int NS>
+cudaError_t fused_x2_prepare_t(const FusedPlan &p, int *blocks_per_sm) {
   using K = FusedK2<LAT, ST, BX, BY, NS>;
+  if (p.rows) {
+    if constexpr (HAS_ROWS<LAT, ST, BX, BY, NS>) {
+      const auto kern = fused_step_kernel_x2<LAT, ST, BX, BY, NS, false, true>;
+      cudaError_t e =
+          cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, K::SMEM);
+      if (e == cudaSuccess && blocks_per_sm)
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, kern, K::NT, K::SMEM);
+      return e;
+    }
+    return cudaErrorInvalidValue;
+  }
   cudaError_t e = cudaFuncSetAttribute(fused_step_kernel_x2<LAT, ST, BX, BY, NS>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, K::SMEM);
   if constexpr (sizeof(typename Storage<ST>::T) == 2) {
@@ -659,6 +761,12 @@ cudaError_t fused_x2_launch_t(const FusedPlan &p, const StepArgs &a, const Fused
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
+  if (p.rows) {
+    if constexpr (HAS_ROWS<LAT, ST, BX, BY, NS>)
+      return cudaLaunchKernelEx(&cfg, fused_step_kernel_x2<LAT, ST, BX, BY, NS, false, true>, tm,
+                                a, p.tiles_x, p.tiles_y, p.zlen);
+    return cudaErrorInvalidValue;
+  }
   if constexpr (sizeof(typename Storage<ST>::T) == 2) {
     if (!(a.debug_flags & 2) && om1_is_16bit<ST>(a.omega_f))  // 2: LBM_DEBUG_CONVERT_BEFORE_FMA
       return cudaLaunchKernelEx(&cfg, fused_step_kernel_x2<LAT, ST, BX, BY, NS, true>, tm, a,
@@ -692,10 +800,10 @@ template <int ST>
 cudaError_t fused_x2_prepare_st(int lat, const FusedPlan &p, int *blocks_per_sm) {
 #define SCLBM_X3(id, bx, by, ns) \
   case id:                       \
-    return fused_x2_prepare_t<D3Q19, ST, bx, by, ns>(blocks_per_sm);
+    return fused_x2_prepare_t<D3Q19, ST, bx, by, ns>(p, blocks_per_sm);
 #define SCLBM_X2(id, bx, by, ns) \
   case id:                       \
-    return fused_x2_prepare_t<D2Q9, ST, bx, by, ns>(blocks_per_sm);
+    return fused_x2_prepare_t<D2Q9, ST, bx, by, ns>(p, blocks_per_sm);
   if (lat == D3Q19) {
     switch (p.tile) { SCLBM_D3Q19_X2_TILES(SCLBM_X3) }
   } else {

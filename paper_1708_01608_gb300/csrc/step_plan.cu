@@ -89,7 +89,7 @@ constexpr TileCost COST_2D_F64[] = {{1, 2.6f, 25.5f, 2.6f, 25.5f}, {3, 2.6f, 25.
 
 template <size_t N>
 cudaError_t pick_plan(const TileCost (&cand)[N], int lat, int st, int64_t NX, int64_t NY,
-                      int64_t NZ, FusedPlan *p) {
+                      int64_t NZ, bool rows, FusedPlan *p) {
   int dev = 0, nsm = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
@@ -102,7 +102,7 @@ cudaError_t pick_plan(const TileCost (&cand)[N], int lat, int st, int64_t NX, in
   bool found = false;
   for (const TileCost &c : cand) {
     FusedPlan q;
-    if (fused_make_plan(lat, st, c.tile, NX, NY, NZ, 1, &q) != cudaSuccess) {
+    if (fused_make_plan(lat, st, c.tile, NX, NY, NZ, 1, &q, rows) != cudaSuccess) {
       cudaGetLastError();
       continue;
     }
@@ -149,16 +149,16 @@ cudaError_t pick_plan(const TileCost (&cand)[N], int lat, int st, int64_t NX, in
 }  // namespace
 
 cudaError_t fused_make_plan(int lat, int st, int tile, int64_t NX, int64_t NY, int64_t NZ,
-                            int nzc, FusedPlan *p) {
+                            int nzc, FusedPlan *p, bool rows) {
   int bx, by, ns, xc;
   if (tile <= 0) {
     if (lat == D2Q9)
-      return st == ST_F64 ? pick_plan(COST_2D_F64, lat, st, NX, NY, NZ, p)
-                          : pick_plan(COST_2D, lat, st, NX, NY, NZ, p);
-    return st == ST_F64   ? pick_plan(COST_F64, lat, st, NX, NY, NZ, p)
-           : st == ST_F32 ? pick_plan(COST_F32, lat, st, NX, NY, NZ, p)
-           : st == ST_F16R || st == ST_BF16R ? pick_plan(COST_H16R, lat, st, NX, NY, NZ, p)
-                                             : pick_plan(COST_H16, lat, st, NX, NY, NZ, p);
+      return st == ST_F64 ? pick_plan(COST_2D_F64, lat, st, NX, NY, NZ, rows, p)
+                          : pick_plan(COST_2D, lat, st, NX, NY, NZ, rows, p);
+    return st == ST_F64   ? pick_plan(COST_F64, lat, st, NX, NY, NZ, rows, p)
+           : st == ST_F32 ? pick_plan(COST_F32, lat, st, NX, NY, NZ, rows, p)
+           : st == ST_F16R || st == ST_BF16R ? pick_plan(COST_H16R, lat, st, NX, NY, NZ, rows, p)
+                                             : pick_plan(COST_H16, lat, st, NX, NY, NZ, rows, p);
   }
   if (!fused_tile_shape(lat, st, tile, &bx, &by, &ns, &xc)) return cudaErrorInvalidValue;
   p->tile = tile;
@@ -169,7 +169,9 @@ cudaError_t fused_make_plan(int lat, int st, int tile, int64_t NX, int64_t NY, i
   p->threads = bx * by / xc;
   p->hx = (int)(16 / storage_bytes(st));
   p->smem = fused_smem_bytes(lat, st, tile, xc);
-  if (NX % p->hx != 0) return cudaErrorInvalidValue;  // halo boxes must start on 16 bytes
+  p->rows = rows;
+  if (rows && xc != 2) return cudaErrorInvalidValue;
+  if (!rows && NX % p->hx != 0) return cudaErrorInvalidValue;  // halo boxes must start on 16 bytes
   int dev = 0, nsm = 0, smem_optin = 0, smem_sm = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;

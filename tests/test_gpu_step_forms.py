@@ -101,11 +101,18 @@ ROWS = [("D3Q19", (1, 1, 1)), ("D3Q19", (1, 9, 4)), ("D3Q19", (29, 6, 3)), ("D3Q
         ("D2Q9", (125, 9, 1)), ("D2Q9", (126, 8, 1)), ("D2Q9", (127, 1500, 1)), ("D2Q9", (255, 2, 1))]
 
 
-@pytest.mark.parametrize("lat,ext", ROWS)
+# enough cells for the x-pair form: tiles (64 x 8, 128 x 4) with one column or
+# row over, an odd and an even last pair, rows narrower than a halo box
+WIDE = [("D3Q19", (129, 33, 150)), ("D3Q19", (65, 57, 170)), ("D3Q19", (130, 9, 520)),
+        ("D3Q19", (127, 40, 120)), ("D3Q19", (201, 150, 21)), ("D3Q19", (1, 800, 760)),
+        ("D3Q19", (3, 460, 450)), ("D3Q19", (600001, 1, 1))]
+
+
+@pytest.mark.parametrize("lat,ext", ROWS + WIDE)
 @pytest.mark.parametrize("storage", ["f32", "f16", "bf16"])
 def test_one_launch_step_gives_the_bits_of_the_two_pass_step(lbm, lat, ext, storage):
     """Rows that are no multiple of 16 bytes, at the edges of the march's
-    tiles (30 x 6 and 126 cells) and chunks: the step an automatic choice
+    tiles (30 x 6 and 126 cells) and chunks and in the x-pair form: the step an automatic choice
     takes there has the populations and budgets of the two-pass kernels, with
     two injection sites in one cell and a neighbouring one."""
     nx, ny, nz = ext
