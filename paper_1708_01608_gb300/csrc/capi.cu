@@ -1018,7 +1018,8 @@ static void count_merges(lbm_ctx *c) {
   c->have_prev = true;
 }
 
-lbm_status lbm_film_probe(lbm_ctx *c, const int64_t *line, double rho_mid, lbm_film *out) {
+static lbm_status film_probe(lbm_ctx *c, const int64_t *line, double rho_mid,
+                             const FilmRule &rule, lbm_film *out) {
   if (!c || !line || !out) return fail(LBM_EINVAL, "NULL argument");
   if (!c->seeded) return fail(LBM_ESTATE, "seed the lattice first");
   const int dims = c->lat == D2Q9 ? 2 : 3;
@@ -1037,13 +1038,12 @@ lbm_status lbm_film_probe(lbm_ctx *c, const int64_t *line, double rho_mid, lbm_f
     z0 = y0;
     y0 = 0;
   }
-  double *tmp = static_cast<double *>(c->d_tmp.p);
+  // the kernel writes its six doubles straight to the pinned mailbox
+  CKS(halloc(c, c->h_mail, 6 * sizeof(double)));
+  double *h = static_cast<double *>(c->h_mail.p);
   CK(diag_film_probe(c->v, static_cast<const double *>(c->d_rho.p),
                      static_cast<const double *>(c->d_p.p), wrap64(x0, c->v.NX), wrap64(y0, c->v.NY),
-                     wrap64(z0, c->v.NZ), e, ep, line[4], rho_mid, tmp, c->s));
-  CKS(halloc(c, c->h_mail, 6 * sizeof(double)));
-  const double *h = static_cast<const double *>(c->h_mail.p);
-  CK(cudaMemcpyAsync(c->h_mail.p, tmp, 6 * sizeof(double), cudaMemcpyDeviceToHost, c->s));
+                     wrap64(z0, c->v.NZ), e, ep, line[4], rho_mid, h, rule, c->s));
   CKS(sync_and_check(c));
   out->found = h[0] != 0.0;
   out->x1 = h[1];
@@ -1052,6 +1052,10 @@ lbm_status lbm_film_probe(lbm_ctx *c, const int64_t *line, double rho_mid, lbm_f
   out->d2p_mid = h[4];
   out->r_d = h[5];
   return LBM_OK;
+}
+
+lbm_status lbm_film_probe(lbm_ctx *c, const int64_t *line, double rho_mid, lbm_film *out) {
+  return film_probe(c, line, rho_mid, FilmRule{}, out);
 }
 
 lbm_status lbm_run_until_rupture(lbm_ctx *c, const int64_t *line, double rho_mid,
@@ -1069,7 +1073,7 @@ lbm_status lbm_run_until_rupture(lbm_ctx *c, const int64_t *line, double rho_mid
     CKS(lbm_step(c, n));
     t += n;
     lbm_film pr;
-    CKS(lbm_film_probe(c, line, rho_mid, &pr));
+    CKS(film_probe(c, line, rho_mid, FilmRule{0, armed, eps_arm, h_max}, &pr));
     out->steps = t;
     if (!pr.found) {  // the film is gone: merged before the criterion fired
       out->merged = 1;

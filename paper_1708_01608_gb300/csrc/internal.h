@@ -249,9 +249,21 @@ cudaError_t diag_label_links(const View &v, int32_t *labels, unsigned long long 
 cudaError_t diag_label(const View &v, const double *rho, double thr, int32_t *labels,
                        unsigned long long *ncomp_dev, cudaStream_t s);
 // film probe along a line (view coordinates, directions e and ep); out: 6 doubles
+// When a film probe wants the disc radius: always, or only where the rupture
+// criterion fires on it (an armed film of at most h_max whose d2p has
+// reached 0).  A run under the probe reports the radius of that one state,
+// and the disc's rows are chains of dependent loads by a single CTA.  A probe
+// in a run, result through a device buffer and a copy / without the disc and
+// straight to pinned memory: 51 / 28 us at 200^2 FP32 (1000 steps with 50
+// probes 6.58 / 5.44 ms); multi-lattice 104^2, 600 steps, 8.75 / 8.15 ms.
+struct FilmRule {
+  int always = 1, armed = 0;
+  double eps_arm = 0, h_max = 0;
+};
+// out (6 doubles) may be pinned host memory
 cudaError_t diag_film_probe(const View &v, const double *rho, const double *p, int64_t x0,
                             int64_t y0, int64_t z0, const int e[3], const int ep[3], int64_t len,
-                            double mid, double *out, cudaStream_t s);
+                            double mid, double *out, const FilmRule &rule, cudaStream_t s);
 cudaError_t diag_gather_labels(const int32_t *labels, const int32_t *cells, int32_t n,
                                int32_t *out, cudaStream_t s);
 // bubble census (census.cu): component sizes from labels (count_scratch: N

@@ -336,6 +336,7 @@ struct lbm_ml_ctx {
   double *d_rho = nullptr, *d_p = nullptr, *d_tmp = nullptr, *d_bub = nullptr;
   double *d_rate = nullptr, *d_budget = nullptr;
   int32_t *d_site = nullptr;  // x, y, z, lattice per site (view coordinates)
+  double *h_mail = nullptr;   // pinned: the film probe's result
   int32_t nsites = 0;
   std::vector<int32_t> site_xyz;
   MlTile tile{};
@@ -627,6 +628,7 @@ void lbm_ml_destroy(lbm_ml_ctx *c) {
   cudaStreamSynchronize(c->s);
   cudaGetLastError();
   ml_free_all(c);
+  if (c->h_mail) cudaFreeHost(c->h_mail);
   delete c;
 }
 
@@ -867,7 +869,8 @@ lbm_status lbm_ml_run_until_rupture(lbm_ml_ctx *c, const int64_t *line, double r
   };
   bool armed = false;
   double h_prev = 0.0, d_prev = 0.0;
-  double h[6];
+  if (!c->h_mail) MLCK(cudaMallocHost(reinterpret_cast<void **>(&c->h_mail), 6 * sizeof(double)));
+  double *h = c->h_mail;
   int64_t t = 0;
   while (t < max_steps) {
     const int64_t n = std::min(diag_every, max_steps - t);
@@ -876,8 +879,7 @@ lbm_status lbm_ml_run_until_rupture(lbm_ml_ctx *c, const int64_t *line, double r
     // the film on the fluid lattice's density, with the coupled pressure
     MLCKS(ml_enqueue_fields(c));
     MLCK(diag_film_probe(c->v, c->d_rho, c->d_p, wr(x0, c->v.NX), wr(y0, c->v.NY), wr(z0, c->v.NZ),
-                         e, ep, line[4], rho_mid, c->d_tmp, c->s));
-    MLCK(cudaMemcpyAsync(h, c->d_tmp, sizeof(h), cudaMemcpyDeviceToHost, c->s));
+                         e, ep, line[4], rho_mid, h, FilmRule{0, armed, eps_arm, h_max}, c->s));
     MLCKS(ml_sync(c));
     out->steps = t;
     const bool found = h[0] != 0.0;
