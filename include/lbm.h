@@ -81,7 +81,7 @@ typedef enum {
 typedef enum {
   LBM_KERNEL_AUTO = 0,    /* fused kernel with the tuned tile */
   LBM_KERNEL_FUSED = 1,   /* one pass: TMA-staged tiles, psi halo in smem */
-  LBM_KERNEL_TWO_PASS = 2 /* psi field pass + collide/stream pass */
+  LBM_KERNEL_TWO_PASS = 2 /* psi field pass + collide/stream pass (AUTO: in one launch, same bits) */
 } lbm_kernel;
 
 /* Optional device allocator.  alloc returns device memory of `bytes` usable
