@@ -85,8 +85,9 @@ template <int LAT, class T>
 struct RelaxK {
   static constexpr T R = LAT == D3Q19 ? 2 : 4;     // axis weight / edge weight
   static constexpr T R0 = LAT == D3Q19 ? 12 : 16;  // rest weight / edge weight
-  T om1, wK, cB;
-  __device__ __forceinline__ RelaxK(T om1_, T wK_, T cB_) : om1(om1_), wK(wK_), cB(cB_) {}
+  T om1, wK, cB, eps;
+  __device__ __forceinline__ RelaxK(T om1_, T wK_, T cB_, T eps_)
+      : om1(om1_), wK(wK_), cB(cB_), eps(eps_) {}
 };
 
 template <int CC, class T>
@@ -123,6 +124,17 @@ __device__ __forceinline__ void pair_moments(Dq dq, T (&m)[3]) {
 
 // The relaxed populations of a cell: f(i) its populations, rho their sum,
 // v = 1.5 u, B = 3 omega w rho u; out(integral_constant i, value).
+//
+// Mass.  The populations together carry om1 + 36 wK of rho, the same wrong
+// factor in every cell and step by the rounding of the two constants, and 36
+// times the rounding of K.  FP64 adds both to the rest population inside its
+// FMA (added after it they would be rounded off): 4 of a cell's 174 FP64
+// instructions.  Total mass after 300 steps against velocity by velocity, rms
+// over 320 runs (D3Q19 and D2Q9, tau 0.6 to 1.4, with and without a bubble):
+// without 1.5e-14, with eps alone 5.0e-15, with both 1.5e-15.  FP32 gives the
+// rest population rho minus the moving ones, as the FP32 step kernels do: of
+// the largest population after 400 steps, velocity by velocity 1.9e-6, from K
+// 1.1e-5, this 7e-8 (two lattices, D2Q9, tau 0.6).
 template <int LAT, class T, class F, class Out>
 __device__ __forceinline__ void relax_pairs(const RelaxK<LAT, T> &q, F f, T rho, const T (&v)[3],
                                             const T (&B)[3], Out out) {
@@ -135,8 +147,16 @@ __device__ __forceinline__ void relax_pairs(const RelaxK<LAT, T> &q, F f, T rho,
     Q[a] = B[a] * v[a];
     s += Q[a];
   }
-  const T K = fma(s, (T)(-1.0 / 3.0), q.wK * rho);
-  out(std::integral_constant<int, 0>{}, fma(q.om1, f(0), R0 * K));
+  const T ts = s * (T)(-1.0 / 3.0), K = fma(q.wK, rho, ts);
+  constexpr bool REST = sizeof(T) == 4;
+  T moved = (T)-0.0;
+  if constexpr (!REST)
+    out(std::integral_constant<int, 0>{},
+        fma(q.om1, f(0), fma(R0, K, fma((T)36, fma(q.wK, rho, ts - K), q.eps * rho))));
+  auto put = [&](auto ic, T x) {
+    if constexpr (REST) moved += x;
+    out(ic, x);
+  };
   static_for<L::NP>([&](auto kc) {
     constexpr int i = L::rep(decltype(kc)::value), o = L::opp(i);
     constexpr int cx = L::cx(i), cy = L::cy(i), cz = L::cz(i);
@@ -144,8 +164,8 @@ __device__ __forceinline__ void relax_pairs(const RelaxK<LAT, T> &q, F f, T rho,
     constexpr int a = cx ? 0 : (cy ? 1 : 2);
     if constexpr (cx * cx + cy * cy + cz * cz == 1) {
       const T A = R * (K + Q[a]);
-      out(std::integral_constant<int, i>{}, fma(R, B[a], fma(q.om1, f(i), A)));
-      out(std::integral_constant<int, o>{}, fma(-R, B[a], fma(q.om1, f(o), A)));
+      put(std::integral_constant<int, i>{}, fma(R, B[a], fma(q.om1, f(i), A)));
+      put(std::integral_constant<int, o>{}, fma(-R, B[a], fma(q.om1, f(o), A)));
     } else {
       constexpr int b = cz ? 2 : 1;
       const T D = (K + Q[a]) + Q[b], v2 = v[b] + v[b];
@@ -153,10 +173,11 @@ __device__ __forceinline__ void relax_pairs(const RelaxK<LAT, T> &q, F f, T rho,
       // c_a B_a + c_b B_b up to the sign of c_a
       const T t = c[a] * c[b] > 0 ? B[a] + B[b] : B[a] - B[b];
       const T hi = fma(q.om1, f(i), A), ho = fma(q.om1, f(o), A);
-      out(std::integral_constant<int, i>{}, c[a] > 0 ? hi + t : hi - t);
-      out(std::integral_constant<int, o>{}, c[a] > 0 ? ho - t : ho + t);
+      put(std::integral_constant<int, i>{}, c[a] > 0 ? hi + t : hi - t);
+      put(std::integral_constant<int, o>{}, c[a] > 0 ? ho - t : ho + t);
     }
   });
+  if constexpr (REST) out(std::integral_constant<int, 0>{}, rho - moved);
 }
 
 // The FP64 collision of one cell.  f(i): its populations, rho their sum,

@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <cmath>
+
 #include "lbm.h"
 
 namespace sclbm {
@@ -16,11 +18,18 @@ lbm_status set_error(lbm_status st, const char *msg);
 // division per thread would cost a tenth of a small lattice's step.
 struct RelaxArgs {
   double om1, wK, cB;   // 1 - omega, omega w, 3 omega w (w = 1/36)
+  // what om1 + 36 wK lacks, by the rounding of the two, of the factor that a step
+  // velocity by velocity puts on a cell's mass: the weights, as FP64 numbers, add
+  // up to 1 - 2^-54 (both lattices), so it is 1 - omega 2^-54
+  double eps;
   double fG, inv_rho0;  // -tau G w, 1/rho0
 };
 inline RelaxArgs make_relax(double tau, double G, double rho0) {
   const double omega = 1.0 / tau, w = 1.0 / 36.0;
-  return RelaxArgs{1.0 - omega, omega * w, 3.0 * omega * w, -tau * G * w, 1.0 / rho0};
+  const double om1 = 1.0 - omega, wK = omega * w;
+  // 1 - om1 is exact (Sterbenz), and so is what the FMA leaves of it
+  const double eps = std::fma(-36.0, wK, 1.0 - om1) - omega * 0x1p-54;
+  return RelaxArgs{om1, wK, 3.0 * omega * w, eps, -tau * G * w, 1.0 / rho0};
 }
 
 // Everything a step kernel needs.  Cells are addressed in the kernels'

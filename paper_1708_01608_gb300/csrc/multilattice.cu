@@ -49,7 +49,7 @@ struct MlArgs {
   int64_t NX, NY, NZ;  // view extents (D2Q9 on (nx, 1, ny))
   int nl;
   T rho0, inv_rho0;
-  T om1, wK, cB, fG;  // RelaxArgs
+  T om1, wK, cB, eps, fG;  // RelaxArgs
   T Gm[ML_MAX * ML_MAX];
 };
 
@@ -147,7 +147,7 @@ __global__ void __launch_bounds__(ML_TPB, sizeof(T) == 8 ? 2 : 3) k_ml_step(cons
   const T *f = static_cast<const T *>(a.fin);
   const int tid = threadIdx.x, x0 = blockIdx.y * tl.tx;
   for (int k = tid; k < ML_MAX * ML_MAX; k += blockDim.x) sG[k] = a.Gm[k];
-  const RelaxK<LAT, T> relax(a.om1, a.wK, a.cB);
+  const RelaxK<LAT, T> relax(a.om1, a.wK, a.cB, a.eps);
   const T rho0 = a.rho0, inv_rho0 = a.inv_rho0;
   const int s = (int)fdiv((uint32_t)tid, tl.fcells, (uint32_t)cells), c = tid - s * cells;
   const int cz_ = FIELD ? 0 : (int)fdiv((uint32_t)c, tl.ftx, (uint32_t)tl.tx);
@@ -443,6 +443,7 @@ MlArgs<T> ml_args(const lbm_ml_ctx *c) {
   a.om1 = (T)r.om1;
   a.wK = (T)r.wK;
   a.cB = (T)r.cB;
+  a.eps = (T)r.eps;
   a.fG = (T)r.fG;
   for (int k = 0; k < ML_MAX * ML_MAX; ++k) a.Gm[k] = (T)c->Gm[k];
   return a;

@@ -316,7 +316,8 @@ __device__ __forceinline__ bool fused_march(const MarchArgs &m, OutPop out_pop, 
     c45[k2] = (C)4.5 * w * omega;
   }
 
-  [[maybe_unused]] const RelaxK<LAT, double> relax(m.relax.om1, m.relax.wK, m.relax.cB);
+  [[maybe_unused]] const RelaxK<LAT, double> relax(m.relax.om1, m.relax.wK, m.relax.cB,
+                                                m.relax.eps);
 
   // two planes per iteration where registers allow (512-thread tiles): the
   // staged values then change register sets instead of being copied

@@ -139,7 +139,7 @@ __global__ void __launch_bounds__(TX *TY, MINB)
       T f[Q];
 #pragma unroll
       for (int i = 0; i < Q; ++i) f[i] = own[i * pop];
-      const RelaxK<LAT, double> relax(a.relax.om1, a.relax.wK, a.relax.cB);
+      const RelaxK<LAT, double> relax(a.relax.om1, a.relax.wK, a.relax.cB, a.relax.eps);
       collide_f64<LAT, false>(
           relax, a.relax.fG, [&](int i) { return f[i]; }, r2, psi_at(0), psi_at,
           [&](auto ic, C v) { *dst(decltype(ic)::value) = v; }, 0.0);
