@@ -87,6 +87,14 @@ __device__ __forceinline__ double psi_f64(double rho, double rho0, double inv_rh
   return fma(-rho0, fma(S, q, S), rho0);
 }
 
+// Whether the reciprocal of b may be infinite: |b| below the normal numbers
+__device__ __forceinline__ bool rcp_overflows(double b) {
+  return (__double2hiint(b) & 0x7fffffff) < 0x00100000;
+}
+__device__ __forceinline__ bool rcp_overflows(float b) {
+  return (__float_as_int(b) & 0x7fffffff) < 0x00800000;
+}
+
 // Density of one cell from its Q values, in two chains (half the latency of
 // one; the owner and a neighbour's halo thread use the same order)
 template <int Q, class Ld>
@@ -220,7 +228,7 @@ __device__ __forceinline__ void collide_f64(const RelaxK<LAT, double> &q, double
   for (int a = 0; a < 3; ++a) {
     if (a == 1 && !L::HAS_Y) continue;
     const double m = fma(gp, s[a], j[a]);
-    v[a] = m * ir;
+    v[a] = rcp_overflows(rho) ? 1.5 * (m / rho) : m * ir;
     B[a] = q.cB * m;
   }
   relax_pairs<LAT, double>(q, f, rho, v, B, [&](auto ic, double x) {

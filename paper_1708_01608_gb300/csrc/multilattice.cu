@@ -86,8 +86,7 @@ __device__ __forceinline__ float ml_rcp(float v) { return 1.0f / v; }
 // where it is finite: a division for every cell cost 2 % of a step (104^2,
 // three lattices).
 __device__ __forceinline__ double ml_quot(double a, double b) {
-  if ((__double2hiint(b) & 0x7fffffff) < 0x00100000) return a / b;  // |b| < 2^-1022
-  return a * __drcp_rn(b);
+  return rcp_overflows(b) ? a / b : a * __drcp_rn(b);
 }
 __device__ __forceinline__ float ml_quot(float a, float b) { return a / b; }
 
@@ -229,7 +228,7 @@ __global__ void __launch_bounds__(ML_TPB, sizeof(T) == 8 ? 2 : 3) k_ml_step(cons
 #pragma unroll
       for (int d = 0; d < 3; ++d) {
         if (d == 1 && !L::HAS_Y) continue;
-        const T u = fma(h, A[d], jt[d] * ir);
+        const T u = fma(h, A[d], rcp_overflows(rt) ? jt[d] / rt : jt[d] * ir);
         v[d] = (T)1.5 * u;
         B[d] = relax.cB * (rho * u);
       }

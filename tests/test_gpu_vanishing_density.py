@@ -73,3 +73,52 @@ def test_one_step_of_vanishing_lattices(lbm, lat, ext, storage):
     want = O.ml_run(LAT[lat], f0, 1, 0.9, O.ml_coupling(nl, -5.0, 1.0, 2.0))
     want = want[0] if isinstance(want, tuple) else want
     assert rel_err(got, want) < 180 * nl * (1.1e-16 if storage == "f64" else 6e-8)
+
+
+@pytest.mark.parametrize("lat,ext", [("D2Q9", (40, 9, 1)), ("D3Q19", (40, 3, 4))])
+@pytest.mark.parametrize("storage", ["f64", "f32"])
+def test_one_step_where_every_lattice_vanishes(lbm, lat, ext, storage):
+    """As above with cells in which the total density is subnormal, whose
+    reciprocal the common velocity must not take."""
+    nx, ny, nz = ext
+    nl, q = 2, 19 if lat == "D3Q19" else 9
+    fi = np.finfo(np.float64 if storage == "f64" else np.float32)
+    tiny = float(fi.smallest_normal)
+    _, w = O.velocities(LAT[lat])
+    rng = np.random.default_rng(4)
+    f0 = (w[None, :, None, None, None] * rng.uniform(0.1, 1.0, size=(nl, 1, nz, ny, nx))
+          * rng.uniform(0.9, 1.1, size=(nl, q, nz, ny, nx)))
+    scale = np.resize([1.0, 1.0, tiny / 4, 1.0, tiny / 2048, 1.0, tiny], (nz, ny, nx))
+    f0 = (f0 * scale).astype(fi.dtype).astype(np.float64)
+    M = lbm.MultiLattice(lat, nx, ny, nz, nl=nl, tau=0.9, G=-5.0, G_x=1.0, G_b=2.0,
+                         storage=storage)
+    M.write_f(f0)
+    M.step(1)
+    got = M.read_f()
+    M.close()
+    assert np.isfinite(got).all()
+    want = O.ml_run(LAT[lat], f0, 1, 0.9, O.ml_coupling(nl, -5.0, 1.0, 2.0))
+    want = want[0] if isinstance(want, tuple) else want
+    assert rel_err(got, want) < 180 * nl * (1.1e-16 if storage == "f64" else 6e-8)
+
+
+@pytest.mark.parametrize("lat,ext", [("D2Q9", (40, 9, 1)), ("D3Q19", (40, 3, 4)),
+                                     ("D2Q9", (41, 9, 1)), ("D3Q19", (41, 3, 4))])
+def test_fp64_step_where_the_density_vanishes(lbm, lat, ext):
+    """The single-component FP64 step (even rows fused, odd ones in one
+    launch) with cells of subnormal density: 40 roundings per population."""
+    nx, ny, nz = ext
+    q = 19 if lat == "D3Q19" else 9
+    tiny = float(np.finfo(np.float64).smallest_normal)
+    _, w = O.velocities(LAT[lat])
+    rng = np.random.default_rng(5)
+    f0 = (w[:, None, None, None] * rng.uniform(0.1, 1.0, size=(1, nz, ny, nx))
+          * rng.uniform(0.9, 1.1, size=(q, nz, ny, nx)))
+    f0 = f0 * np.resize([1.0, 1.0, tiny / 4, 1.0, tiny / 2048, 1.0, tiny], (nz, ny, nx))
+    L = lbm.Lattice(lat, nx, ny, nz, tau=0.8, G=-5.0, storage="f64")
+    L.write_f(f0)
+    L.step(1)
+    got = L.read("f")
+    L.close()
+    assert np.isfinite(got).all()
+    assert rel_err(got, O.run(LAT[lat], f0, 1, 0.8, -5.0)) < 2e-14
