@@ -10,7 +10,6 @@
 #include <cstring>
 #include <map>
 #include <string>
-#include <system_error>
 #include <thread>
 #include <vector>
 
@@ -275,7 +274,7 @@ void back_pages(void *dst, size_t bytes) {
   size_t started = 1;
   try {
     for (; started < n; ++started) team[started] = std::thread(back, started);
-  } catch (const std::system_error &) {  // no more threads: the copy does the rest
+  } catch (...) {  // no thread, or no memory for one: the copy does the rest
   }
   back(0);
   for (size_t k = 1; k < started; ++k) team[k].join();
