@@ -576,7 +576,7 @@ __device__ __forceinline__ bool fused_march_x2(const MarchArgs &m, OutPop out_po
           static_assert(L::HAS_Y, "opposite velocities are neighbours in the order of the sum");
           static_for<L::NP>([&](auto kc) {
             constexpr int i = L::rep(decltype(kc)::value), o = L::opp(i);
-                        const float2 cu = cdot2<L::cx(i), L::cy(i), L::cz(i)>(ux, uy, uz);
+            const float2 cu = cdot2<L::cx(i), L::cy(i), L::cz(i)>(ux, uy, uz);
             const float2 q = mul2(mul2(f2(4.5f), cu), cu);
             auto relax = [&](float2 e, float2 g) {
               const float2 t = fma2(f2(-(float)L::w(i)), fma2(rho, e, Kc), g);
@@ -590,80 +590,80 @@ __device__ __forceinline__ bool fused_march_x2(const MarchArgs &m, OutPop out_po
           });
           put(std::integral_constant<int, 0>{}, sub2(R, moved));
         } else {
-        float2 jx = f2(-0.0f), jy = f2(-0.0f), jz = f2(-0.0f);
-        float2 sx = f2(-0.0f), sy = f2(-0.0f), sz = f2(-0.0f);
-        static_for<L::NP>([&](auto kc) {
-          constexpr int k2 = decltype(kc)::value, i = L::rep(k2), o = L::opp(i);
-          constexpr int cx = L::cx(i), cy = L::cy(i), cz = L::cz(i);
-          float2 d;
-          if constexpr (sizeof(T) == 2) {
-            const float2 vo = S2::load(cur[o]);
-            d = make_float2(sub_w(lo16(cur[i]), vo.x), sub_w(hi16(cur[i]), vo.y));
-          } else {
-            d = sub2(S2::load(cur[i]), S2::load(cur[o]));
-          }
-          jx = cacc2<cx>(jx, d);
-          jy = cacc2<cy>(jy, d);
-          jz = cacc2<cz>(jz, d);
-          const float2 dps = sub2(psi2_at(std::integral_constant<int, i>{}),
-                                  psi2_at(std::integral_constant<int, o>{}));
-          const float w = (float)L::w(i);
-          sx = cfma2<cx>(sx, w, dps);
-          sy = cfma2<cy>(sy, w, dps);
-          sz = cfma2<cz>(sz, w, dps);
-        });
-        const float2 rho = add2(f2(rho_ref), R);
-        const float2 gp = mul2(f2(-G), *reinterpret_cast<const float2 *>(ringN + k0p * RP + c0));
-        const float2 ir = make_float2(__fdividef(1.0f, rho.x), __fdividef(1.0f, rho.y));
-        const float2 ux = mul2(fma2(f2(tau), mul2(gp, sx), jx), ir);
-        const float2 uy = mul2(fma2(f2(tau), mul2(gp, sy), jy), ir);
-        const float2 uz = mul2(fma2(f2(tau), mul2(gp, sz), jz), ir);
-        const float2 uu = fma2(uz, uz, fma2(uy, uy, mul2(ux, ux)));
-        const float2 Kc = fma2(mul2(rho, f2(-1.5f)), uu, R);
-        const float2 wK[2] = {mul2(f2(cW[0]), Kc), mul2(f2(cW[1]), Kc)};
-        const float2 om1_2 = f2(om1);
-        [[maybe_unused]] T om1h;
-        if constexpr (OM16) om1h = S1::store(om1);
-        // relax and push (offset form, as in the one-cell march):
-        //   g_i* = (1 - omega) g_i + omega w_i (K + 4.5 rho (c.u)^2) + 3 omega w_i rho c.u
-        // SITE adds w_i dm to every population of the site cell
-        auto relax_push = [&](auto with_site) {
-          constexpr bool SITE = decltype(with_site)::value;
-          float2 moved = f2(-0.0f);
+          float2 jx = f2(-0.0f), jy = f2(-0.0f), jz = f2(-0.0f);
+          float2 sx = f2(-0.0f), sy = f2(-0.0f), sz = f2(-0.0f);
           static_for<L::NP>([&](auto kc) {
             constexpr int k2 = decltype(kc)::value, i = L::rep(k2), o = L::opp(i);
-            constexpr int wc = L::w(i) == L::w(L::rep(0)) ? 0 : 1;
-            const float2 cu = cdot2<L::cx(i), L::cy(i), L::cz(i)>(ux, uy, uz);
-            const float2 a = mul2(rho, cu);
-            const float2 A = fma2(a, mul2(f2(c45[wc]), cu), wK[wc]);
-            // A +- B with B = 3 omega w_i a, as FMAs (the one-cell march's form)
-            const float2 Ai = fma2(f2(c3[wc]), a, A), Ao = fma2(f2(-c3[wc]), a, A);
-            float2 gi, go;
-            if constexpr (OM16) {
-              gi = make_float2(fma_w(om1h, lo16(cur[i]), Ai.x), fma_w(om1h, hi16(cur[i]), Ai.y));
-              go = make_float2(fma_w(om1h, lo16(cur[o]), Ao.x), fma_w(om1h, hi16(cur[o]), Ao.y));
+            constexpr int cx = L::cx(i), cy = L::cy(i), cz = L::cz(i);
+            float2 d;
+            if constexpr (sizeof(T) == 2) {
+              const float2 vo = S2::load(cur[o]);
+              d = make_float2(sub_w(lo16(cur[i]), vo.x), sub_w(hi16(cur[i]), vo.y));
             } else {
-              gi = fma2(om1_2, S2::load(cur[i]), Ai);
-              go = fma2(om1_2, S2::load(cur[o]), Ao);
+              d = sub2(S2::load(cur[i]), S2::load(cur[o]));
             }
-            moved = add2(moved, add2(gi, go));
-            if (SITE) {
-              put(std::integral_constant<int, i>{}, fma2(f2((float)L::w(i)), dmc, gi));
-              put(std::integral_constant<int, o>{}, fma2(f2((float)L::w(o)), dmc, go));
-            } else {
-              put(std::integral_constant<int, i>{}, gi);
-              put(std::integral_constant<int, o>{}, go);
-            }
+            jx = cacc2<cx>(jx, d);
+            jy = cacc2<cy>(jy, d);
+            jz = cacc2<cz>(jz, d);
+            const float2 dps = sub2(psi2_at(std::integral_constant<int, i>{}),
+                                    psi2_at(std::integral_constant<int, o>{}));
+            const float w = (float)L::w(i);
+            sx = cfma2<cx>(sx, w, dps);
+            sy = cfma2<cy>(sy, w, dps);
+            sz = cfma2<cz>(sz, w, dps);
           });
-          const float2 g0 = sub2(R, moved);
-          put(std::integral_constant<int, 0>{},
-              SITE ? fma2(f2((float)L::w(0)), dmc, g0) : g0);
-        };
-        if (site)
-          relax_push(std::true_type{});
-        else
-          relax_push(std::false_type{});
-        if constexpr (RESID) *reinterpret_cast<float2 *>(m.resid + own) = racc;
+          const float2 rho = add2(f2(rho_ref), R);
+          const float2 gp = mul2(f2(-G), *reinterpret_cast<const float2 *>(ringN + k0p * RP + c0));
+          const float2 ir = make_float2(__fdividef(1.0f, rho.x), __fdividef(1.0f, rho.y));
+          const float2 ux = mul2(fma2(f2(tau), mul2(gp, sx), jx), ir);
+          const float2 uy = mul2(fma2(f2(tau), mul2(gp, sy), jy), ir);
+          const float2 uz = mul2(fma2(f2(tau), mul2(gp, sz), jz), ir);
+          const float2 uu = fma2(uz, uz, fma2(uy, uy, mul2(ux, ux)));
+          const float2 Kc = fma2(mul2(rho, f2(-1.5f)), uu, R);
+          const float2 wK[2] = {mul2(f2(cW[0]), Kc), mul2(f2(cW[1]), Kc)};
+          const float2 om1_2 = f2(om1);
+          [[maybe_unused]] T om1h;
+          if constexpr (OM16) om1h = S1::store(om1);
+          // relax and push (offset form, as in the one-cell march):
+          //   g_i* = (1 - omega) g_i + omega w_i (K + 4.5 rho (c.u)^2) + 3 omega w_i rho c.u
+          // SITE adds w_i dm to every population of the site cell
+          auto relax_push = [&](auto with_site) {
+            constexpr bool SITE = decltype(with_site)::value;
+            float2 moved = f2(-0.0f);
+            static_for<L::NP>([&](auto kc) {
+              constexpr int k2 = decltype(kc)::value, i = L::rep(k2), o = L::opp(i);
+              constexpr int wc = L::w(i) == L::w(L::rep(0)) ? 0 : 1;
+              const float2 cu = cdot2<L::cx(i), L::cy(i), L::cz(i)>(ux, uy, uz);
+              const float2 a = mul2(rho, cu);
+              const float2 A = fma2(a, mul2(f2(c45[wc]), cu), wK[wc]);
+              // A +- B with B = 3 omega w_i a, as FMAs (the one-cell march's form)
+              const float2 Ai = fma2(f2(c3[wc]), a, A), Ao = fma2(f2(-c3[wc]), a, A);
+              float2 gi, go;
+              if constexpr (OM16) {
+                gi = make_float2(fma_w(om1h, lo16(cur[i]), Ai.x), fma_w(om1h, hi16(cur[i]), Ai.y));
+                go = make_float2(fma_w(om1h, lo16(cur[o]), Ao.x), fma_w(om1h, hi16(cur[o]), Ao.y));
+              } else {
+                gi = fma2(om1_2, S2::load(cur[i]), Ai);
+                go = fma2(om1_2, S2::load(cur[o]), Ao);
+              }
+              moved = add2(moved, add2(gi, go));
+              if (SITE) {
+                put(std::integral_constant<int, i>{}, fma2(f2((float)L::w(i)), dmc, gi));
+                put(std::integral_constant<int, o>{}, fma2(f2((float)L::w(o)), dmc, go));
+              } else {
+                put(std::integral_constant<int, i>{}, gi);
+                put(std::integral_constant<int, o>{}, go);
+              }
+            });
+            const float2 g0 = sub2(R, moved);
+            put(std::integral_constant<int, 0>{},
+                SITE ? fma2(f2((float)L::w(0)), dmc, g0) : g0);
+          };
+          if (site)
+            relax_push(std::true_type{});
+          else
+            relax_push(std::false_type{});
+          if constexpr (RESID) *reinterpret_cast<float2 *>(m.resid + own) = racc;
         }
       }
     }
