@@ -120,6 +120,11 @@ namespace {
 // form: FP32 49^3 7.7 / 10.2, 65^3 13.8 / 18.6, 81^3 22.2 / 24.7, 99^3 43.0 /
 // 35.3, 127^3 80 / 58; FP16 65^3 13.7 / 14.9, 81^3 22.1 / 20.4, 127^3 68 / 44.
 constexpr int64_t kRowsMinCells = 600000;
+// And only where its tiles stage less than this many cells per cell: on
+// narrower lattices march_launch's forms are the faster ones (us per step, FP32,
+// x-pair form / those: 31x8x8065, 2.1 cells, 89 / 100; 9x471x471, 7, 354 / 158;
+// 3x816x816, 21, 991 / 207).
+constexpr double kRowsMaxStaged = 3.0;
 
 void hfree(PinBuf &b) {
   if (b.p) cudaFreeHost(b.p);
@@ -443,8 +448,11 @@ lbm_status lbm_create(const lbm_config *cfg, lbm_ctx **out) {
       c->kernel = LBM_KERNEL_TWO_PASS;
       if (!c->resid && c->lat == D3Q19 && c->st != LBM_F64 && cfg->tile <= 0 &&
           c->N >= kRowsMinCells) {
+        const FusedPlan &p = c->plan;
         c->rows = fused_make_plan(c->lat, c->st_step, 0, c->v.NX, c->v.NY, c->v.NZ, 0, &c->plan,
-                                  true) == cudaSuccess;
+                                  true) == cudaSuccess &&
+                  (double)(p.tiles_x * p.bx) * (double)(p.tiles_y * p.by) * (double)(p.zlen + 2) <
+                      kRowsMaxStaged * (double)(c->v.NX * c->v.NY) * (double)p.zlen;
         cudaGetLastError();
       }
       c->march = !c->resid && !c->rows;
