@@ -92,12 +92,15 @@ __device__ __forceinline__ float ml_quot(float a, float b) { return a / b; }
 
 // What the step kernels need beside MlArgs: the work split (ml_tile).  A CTA
 // takes tx x tz cells of every lattice, one thread per (cell, lattice); on the
-// field form tz is 1 and a CTA row y, z comes from the grid.
+// field form tx cells of a row or, where rows would leave threads idle, tx that
+// follow one another in memory.
 struct MlTile {
   int tx, tz;       // cells of a CTA along x and along the view's z (D2Q9)
+  int hx;           // 1: the psi tile has a halo along x; 0: tx is the whole row
+  int row;          // field form: 1: cells of one row (ML_ROW), else ML_RUN
   int threads, smem;
   unsigned gx, gy;  // grid
-  FastDiv fcells, ftx, fpw, fny;  // by tx tz, tx, tx + 2, NY
+  FastDiv fcells, ftx, fpw, fnx, fny;  // by tx tz, tx, tx + 2 hx, NX, NY
 };
 
 // psi of every lattice into a field, one thread per (cell, lattice): D3Q19,
@@ -128,16 +131,19 @@ __global__ void __launch_bounds__(TPB) k_ml_psi(const MlArgs<T> a, T *psi) {
 // / 11.8, 500^2 698 / 208, D3Q19 64x64x48 912 / 239; FP32 104^2 16.4 / 3.7,
 // 1000^2 161 / 118, 64x64x48 66.6 / 27.2.
 //
-// FIELD: psi comes from k_ml_psi (D3Q19).  Otherwise (D2Q9) the CTA forms it
-// for its tile and a one-cell halo in shared memory, one launch per step.
-template <int LAT, class T, bool FIELD>
+// Forms: psi of the tile and a one-cell halo formed in shared memory, one launch
+// per step (ML_TILE, D2Q9); psi from k_ml_psi, the CTA's cells of one row
+// (ML_ROW) or in memory order (ML_RUN; D3Q19).
+enum { ML_TILE = 0, ML_ROW = 1, ML_RUN = 2 };
+template <int LAT, class T, int FORM>
 __global__ void __launch_bounds__(ML_TPB, sizeof(T) == 8 ? 2 : 3) k_ml_step(const MlArgs<T> a, const MlTile tl,
                                                  const T *psi_field) {
   using L = Lattice<LAT>;
   constexpr int Q = L::Q;
+  constexpr bool FIELD = FORM != ML_TILE;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int nl = a.nl, cells = tl.tx * tl.tz;
-  const int PW = tl.tx + 2, PC = FIELD ? 0 : PW * (tl.tz + 2);
+  const int PW = tl.tx + 2 * tl.hx, PC = FIELD ? 0 : PW * (tl.tz + 2);
   T *sG = reinterpret_cast<T *>(smem_raw);  // coupling matrix
   T *mom = sG + ML_MAX * ML_MAX;            // [lattice][rho, j (3), S (3)][cell]
   T *psis = mom + nl * 7 * cells;           // [lattice][PC]
@@ -151,22 +157,32 @@ __global__ void __launch_bounds__(ML_TPB, sizeof(T) == 8 ? 2 : 3) k_ml_step(cons
   const int s = (int)fdiv((uint32_t)tid, tl.fcells, (uint32_t)cells), c = tid - s * cells;
   const int cz_ = FIELD ? 0 : (int)fdiv((uint32_t)c, tl.ftx, (uint32_t)tl.tx);
   const int cx_ = c - cz_ * tl.tx;
-  const int x = x0 + cx_;
+  int x = x0 + cx_;
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
   const T *fs = f + (int64_t)s * Q * N;
-  const uint32_t rows = FIELD ? (uint32_t)(a.NY * a.NZ) : 1u;
-  for (uint32_t row = FIELD ? blockIdx.x : 0; row < rows; row += gridDim.x) {
-    const int z0 = FIELD ? (int)fdiv(row, tl.fny, (uint32_t)NY) : (int)blockIdx.x * tl.tz;
-    const int y = FIELD ? (int)(row - (uint32_t)z0 * (uint32_t)NY) : 0, z = z0 + cz_;
+  const uint32_t rows = FORM == ML_ROW ? (uint32_t)(a.NY * a.NZ) : gridDim.x;
+  for (uint32_t row = FIELD ? blockIdx.x : 0; row < (FIELD ? rows : 1u); row += gridDim.x) {
+    int z0, y;
+    if constexpr (FORM == ML_RUN) {  // a run of cells; a lattice has fewer than 2^32
+      const uint32_t k = (uint32_t)min((uint64_t)row * (uint64_t)cells + (uint64_t)c, (uint64_t)N);
+      const uint32_t r = fdiv(k, tl.fnx, (uint32_t)NX);
+      x = (int)(k - r * (uint32_t)NX);
+      z0 = (int)fdiv(r, tl.fny, (uint32_t)NY);  // NZ past the last cell
+      y = (int)(r - (uint32_t)z0 * (uint32_t)NY);
+    } else {
+      z0 = FIELD ? (int)fdiv(row, tl.fny, (uint32_t)NY) : (int)blockIdx.x * tl.tz;
+      y = FIELD ? (int)(row - (uint32_t)z0 * (uint32_t)NY) : 0;
+    }
+    const int z = z0 + cz_;
     const bool on = s < nl && x < NX && z < NZ;
     if constexpr (!FIELD) {
       if (s < nl)
         for (int r = c; r < PC; r += cells) {
           const int rz = (int)fdiv((uint32_t)r, tl.fpw, (uint32_t)PW);
           // cells past a ragged tile's halo are not read by anyone
-          const int hx = x0 + r - rz * PW - 1, hz = z0 + rz - 1;
+          const int hx = x0 + r - rz * PW - tl.hx, hz = z0 + rz - 1;
           if (hx > NX || hz > NZ) continue;
           const uint32_t k = (uint32_t)wrapv(hz, NZ) * (uint32_t)NX + (uint32_t)wrapv(hx, NX);
           psis[s * PC + r] = ml_psi_fast(ml_rho<Q>(fs + k, N), rho0, inv_rho0);
@@ -188,9 +204,11 @@ __global__ void __launch_bounds__(ML_TPB, sizeof(T) == 8 ? 2 : 3) k_ml_step(cons
       for (int i = 0; i < Q; ++i) fi[i] = fs[i * N + nb[0]];
       rho = rho_f64<Q>([&](int i) { return fi[i]; });
       const T *pf = FIELD ? psi_field + (int64_t)s * N
-                          : psis + s * PC + (cz_ + 1) * PW + cx_ + 1;
+                          : psis + s * PC + (cz_ + 1) * PW + cx_ + tl.hx;
+      const int xm = tl.hx || cx_ > 0 ? -1 : NX - 1, xp = tl.hx || cx_ + 1 < NX ? 1 : 1 - NX;
       auto psi = [&](int i) -> T {
-        return FIELD ? pf[nb[i]] : pf[L::cz(i) * PW + L::cx(i)];
+        return FIELD ? pf[nb[i]]
+                     : pf[L::cz(i) * PW + (L::cx(i) > 0 ? xp : (L::cx(i) < 0 ? xm : 0))];
       };
       psi0 = psi(0);
       T j[3], S[3];
@@ -237,7 +255,7 @@ __global__ void __launch_bounds__(ML_TPB, sizeof(T) == 8 ? 2 : 3) k_ml_step(cons
           relax, [&](int i) { return fi[i]; }, rho, v, B,
           [&](auto ic, T val) { g[decltype(ic)::value * N + nb[decltype(ic)::value]] = val; });
     }
-    if (FIELD) __syncthreads();  // the moments are read before the next row writes them
+    if (FORM == ML_ROW) __syncthreads();  // the moments are read before the next row writes them
   }
 }
 
@@ -466,8 +484,8 @@ void ml_launch(const lbm_ml_ctx *c, dim3 grid, int threads, int smem, void (*k)(
 
 // The tile of the step kernel.  D2Q9: the tx x tz with the least work on the
 // busiest SM, a cell counting 5 (collision) and a halo position 1 (psi), plus
-// 40 for the launch's fixed latency per CTA.  D3Q19: 64 cells of a row (32
-// from five lattices on).
+// 40 for the launch's fixed latency per CTA.  D3Q19: 64 cells (32 from five
+// lattices on).
 MlTile ml_tile(int lat, int nl, int ts, int64_t NX, int64_t NY, int64_t NZ, int nsm) {
   MlTile best{};
   auto fill = [&](MlTile &t) {
@@ -475,21 +493,34 @@ MlTile ml_tile(int lat, int nl, int ts, int64_t NX, int64_t NY, int64_t NZ, int 
     t.threads = (cells * nl + 31) / 32 * 32;
     t.fcells = make_fastdiv((uint32_t)cells);
     t.ftx = make_fastdiv((uint32_t)t.tx);
-    t.fpw = make_fastdiv((uint32_t)t.tx + 2);
+    t.hx = t.tx < NX || t.tx > NX;
+    t.fpw = make_fastdiv((uint32_t)(t.tx + 2 * t.hx));
+    t.fnx = make_fastdiv((uint32_t)NX);
     t.fny = make_fastdiv((uint32_t)NY);
-    t.smem = ts * (ML_MAX * ML_MAX + nl * (7 * cells + (lat == D2Q9 ? (t.tx + 2) * (t.tz + 2) : 0)));
+    t.smem = ts * (ML_MAX * ML_MAX +
+                   nl * (7 * cells + (lat == D2Q9 ? (t.tx + 2 * t.hx) * (t.tz + 2) : 0)));
   };
   if (lat == D3Q19) {
     best.tx = nl > 4 ? 32 : 64;
     best.tz = 1;
-    best.gx = (unsigned)std::min<int64_t>(NY * NZ, 1 << 30);
-    best.gy = (unsigned)((NX + best.tx - 1) / best.tx);
+    // Rows where they keep 0.8 of the threads busy, in FP64 0.9 of the lanes of
+    // the warps that have any (an idle warp costs the pipe nothing); elsewhere
+    // cells in memory order, whose two more divisions cost 10 % of an FP32 step
+    // on full rows.  us per step, rows / memory order, FP32, one lattice: 1x707x707
+    // 781 / 26, 33x8x1894 34 / 26, 64x977x8 22 / 25.
+    const int64_t unit = ts == 8 ? 32 : best.tx;
+    best.row = NY * NZ <= INT32_MAX &&
+               (double)NX >= (ts == 8 ? 0.9 : 0.8) * (double)((NX + unit - 1) / unit * unit);
+    best.gx = (unsigned)(best.row ? NY * NZ : (NX * NY * NZ + best.tx - 1) / best.tx);
+    best.gy = best.row ? (unsigned)((NX + best.tx - 1) / best.tx) : 1;
     fill(best);
     return best;
   }
   double cost = 0;
-  for (int tx = 8; tx <= 64; tx += 8)
-    for (int tz = 1; tz <= 32; ++tz) {
+  for (int tx0 = 0; tx0 <= 64; tx0 += 8)
+    for (int tz = 1; tz <= std::max(32, ML_TPB / std::max(tx0, 1)); ++tz) {
+      if (tx0 == 0 && NX > 64) break;
+      const int tx = tx0 == 0 ? (int)NX : tx0;  // first: whole rows
       MlTile t{};
       t.tx = tx;
       t.tz = tz;
@@ -497,11 +528,11 @@ MlTile ml_tile(int lat, int nl, int ts, int64_t NX, int64_t NY, int64_t NZ, int 
       const int64_t gx = (NZ + tz - 1) / tz, gy = (NX + tx - 1) / tx;
       if (t.threads > ML_TPB || t.smem > 48 * 1024 || gy > 65535) continue;
       // beyond a few tiles per SM rows of whole 128-byte lines
-      if (gx * gy > 4 * nsm && tx * ts < 128) continue;
+      if (gx * gy > 4 * nsm && tx * ts < 128 && tx < NX) continue;
       t.gx = (unsigned)gx;
       t.gy = (unsigned)gy;
       const double w = (double)((gx * gy + nsm - 1) / nsm) *
-                       (5.0 * tx * tz + (double)(tx + 2) * (tz + 2) + 40.0);
+                       (5.0 * tx * tz + (double)(tx + 2 * t.hx) * (tz + 2) + 40.0);
       if (best.tx == 0 || w < cost) {
         cost = w;
         best = t;
@@ -792,8 +823,17 @@ lbm_status lbm_ml_step(lbm_ml_ctx *c, int64_t nsteps) {
       if constexpr (lat == D3Q19)
         ml_launch(c, dim3((unsigned)nblocks(c->N), (unsigned)c->nl), TPB, 0, k_ml_psi<lat, TT>, a,
                   psi);
-      ml_launch(c, dim3(c->tile.gx, c->tile.gy), c->tile.threads, c->tile.smem,
-                  k_ml_step<lat, TT, lat == D3Q19>, a, c->tile, static_cast<const TT *>(psi));
+      auto step = [&](auto form) {
+        ml_launch(c, dim3(c->tile.gx, c->tile.gy), c->tile.threads, c->tile.smem,
+                  k_ml_step<lat, TT, decltype(form)::value>, a, c->tile,
+                  static_cast<const TT *>(psi));
+      };
+      if constexpr (lat == D2Q9)
+        step(std::integral_constant<int, ML_TILE>{});
+      else if (c->tile.row)
+        step(std::integral_constant<int, ML_ROW>{});
+      else
+        step(std::integral_constant<int, ML_RUN>{});
     });
     if (e == cudaSuccess && c->nsites > 0) e = ml_dispatch(c, [&](auto L, auto T) {
       using TT = decltype(T);

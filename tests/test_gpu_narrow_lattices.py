@@ -6,7 +6,8 @@ import time
 import numpy as np
 import pytest
 
-from helpers import lbm_mod
+import oracle as O
+from helpers import LAT, lbm_mod, rel_err
 
 pytestmark = pytest.mark.gpu
 
@@ -102,3 +103,48 @@ def test_static_step_on_narrow_lattices(lbm, ext):
     n = round((ext[0] * ext[1] * ext[2]) ** (1 / 3))
     t, cube = per_step(*ext), per_step(n, n, n)
     assert t < 3 * cube, (t, cube)
+
+
+@pytest.mark.parametrize("lat,ext,nl", [
+    ("D2Q9", (1, 300, 1), 3), ("D2Q9", (5, 211, 1), 8), ("D2Q9", (9, 1200, 1), 2),
+    ("D2Q9", (63, 65, 1), 4), ("D2Q9", (64, 40, 1), 1), ("D3Q19", (1, 40, 9), 3),
+    ("D3Q19", (3, 21, 30), 8), ("D3Q19", (67, 3, 5), 2), ("D3Q19", (130, 2, 3), 5)])
+@pytest.mark.parametrize("storage", ["f64", "f32"])
+def test_multi_lattice_tiles_of_whole_rows(lbm, lat, ext, nl, storage):
+    """One multi-lattice step where a tile takes whole rows (D2Q9) and on runs
+    of cells that cross rows (D3Q19): 180 u nl of the largest population, as
+    for the tiles of the step."""
+    nx, ny, nz = ext
+    q = 19 if lat == "D3Q19" else 9
+    _, w = O.velocities(LAT[lat])
+    rng = np.random.default_rng(nl)
+    f0 = (w[None, :, None, None, None] * rng.uniform(0.1, 1.0, size=(nl, 1, nz, ny, nx))
+          * rng.uniform(0.9, 1.1, size=(nl, q, nz, ny, nx)))
+    if storage == "f32":
+        f0 = f0.astype(np.float32).astype(np.float64)
+    M = lbm.MultiLattice(lat, nx, ny, nz, nl=nl, tau=0.9, G=-5.0, G_x=1.0, G_b=2.0,
+                         storage=storage)
+    M.write_f(f0)
+    M.step(1)
+    got = M.read_f()
+    M.close()
+    want = O.ml_run(LAT[lat], f0, 1, 0.9, O.ml_coupling(nl, -5.0, 1.0, 2.0))
+    want = want[0] if isinstance(want, tuple) else want
+    assert rel_err(got, want) < 180 * nl * (1.1e-16 if storage == "f64" else 6e-8)
+
+
+@pytest.mark.parametrize("lat,ext,cube", [
+    ("D3Q19", (1, 300, 300), (45, 45, 44)), ("D3Q19", (3, 20000, 3), (57, 57, 55)),
+    ("D2Q9", (1, 160000, 1), (400, 400, 1)), ("D2Q9", (9, 30000, 1), (520, 520, 1))])
+@pytest.mark.parametrize("nl,storage", [(1, "f32"), (3, "f32"), (3, "f64")])
+def test_multi_lattice_step_on_narrow_lattices(lbm, lat, ext, cube, nl, storage):
+    """No more than three times as long as a square or cube of about as many
+    cells (2 to 16 times where most threads idle)."""
+    import torch
+    t = []
+    for e in (ext, cube):
+        M = lbm.MultiLattice(lat, *e, nl=nl, tau=0.9, storage=storage)
+        M.seed([[1.0, 1.0, 0.0, 1.0]] * (nl - 1), 1.8, 0.15, 0.05, 2.0, 1e-3, 5)
+        t.append(_time(M.step, torch.cuda.synchronize))
+        M.close()
+    assert t[0] < 3 * t[1], t
