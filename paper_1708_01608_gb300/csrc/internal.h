@@ -93,7 +93,8 @@ struct FusedPlan {
 // storage.  *xc (may be NULL) receives the cells per thread along x.
 bool fused_tile_shape(int lat, int st, int tile, int *bx, int *by, int *nstage,
                       int *xc = nullptr);
-// Fill *plan for a lattice.  nzc > 0: that many z chunks; 0: the number
+// Fill *plan for a lattice.  tile <= 0: the tile and chunk count of the cost
+// model (nzc is not read).  Else nzc > 0: that many z chunks; 0: the number
 // with the fewest staged planes per resident CTA slot when the CTAs run in
 // waves of SMs x CTAs per SM; -1: as many as fill those slots once.  Returns
 // cudaErrorInvalidValue when the tile does not fit or nx is not a multiple

@@ -87,6 +87,61 @@ constexpr TileCost COST_2D[] = {{4, 0.35f, 0.5f, 0.35f, 0.5f}, {6, 0.35f, 0.6f, 
 // D2Q9 FP64: 64^2 21.1 / 8.8, 128^2 22.0 / 9.2, 512^2 60 / 54
 constexpr TileCost COST_2D_F64[] = {{1, 2.6f, 25.5f, 2.6f, 25.5f}, {3, 2.6f, 25.5f, 2.6f, 25.5f}};
 
+// Narrow lattices with D3Q19 and FP32 arithmetic: rows of 4 to 48 cells, fewer
+// than 8 rows, in FP32 also up to 8 planes.  The copies of a box go row by row
+// and the columns past the lattice are filled in, so that a plane takes nearly
+// as long as a full one, which the model above, in cells of the lattice, does
+// not know (8x250000x1 FP32: its plan, tile 14, 975 us, tile 1 437).  There its
+// plan is compared with tile 1 and the chunks of lbm_config.tile = 1 in a second
+// model: a plane takes max(floor, base + co row rows) us, rows the box's rows in
+// the lattice and its two halo rows, the two halo planes count as `planes`
+// planes, and a CTA takes start us besides.  Fitted to 6700 times on 591 such
+// lattices (rms 7 to 14 %; the tiles then scaled by up to 14 % for the choice).
+// Time against the better of the two plans, first model alone / now, mean and
+// largest: FP32 1.13, 2.23 / 1.01, 1.17; 16-bit 1.06, 1.56 / 1.01, 1.09.
+struct RowCost {
+  int tile;
+  float start, base, row, planes, floor;
+};
+constexpr RowCost ROW_F32[] = {{1, 2.92f, 0.840f, 0.0432f, 0.00f, 0.49f},
+                               {2, 1.69f, 0.524f, 0.0646f, 0.87f, 0.84f},
+                               {14, 1.70f, 0.952f, 0.0590f, 1.18f, 1.17f},
+                               {16, 0.55f, 0.348f, 0.0500f, 2.47f, 1.02f},
+                               {25, 3.02f, 0.754f, 0.0591f, 0.11f, 0.99f}};
+constexpr RowCost ROW_H16[] = {{1, 1.31f, 1.168f, 0.0524f, 1.14f, 1.32f},
+                               {2, 0.15f, 0.711f, 0.0465f, 2.81f, 0.94f},
+                               {23, 1.73f, 0.738f, 0.0674f, 1.01f, 1.03f},
+                               {24, 2.71f, 0.823f, 0.0558f, 0.41f, 0.66f}};
+constexpr RowCost ROW_H16R[] = {{1, 1.41f, 1.232f, 0.0606f, 0.96f, 1.50f},
+                                {2, 0.00f, 0.904f, 0.0487f, 2.42f, 1.15f},
+                                {23, 1.00f, 0.983f, 0.0734f, 1.06f, 1.35f},
+                                {24, 0.01f, 0.277f, 0.1149f, 1.91f, 1.60f}};
+
+// us of a plan in that model; < 0: the tile is not in it
+template <size_t N>
+double row_us(const RowCost (&cand)[N], const FusedPlan &q, int st, int64_t NX, int64_t NY,
+              int64_t NZ, int nsm) {
+  int per_sm = 0;
+  if (fused_prepare(D3Q19, st, q, &per_sm) != cudaSuccess || per_sm < 1) {
+    cudaGetLastError();
+    return -1.0;
+  }
+  for (const RowCost &c : cand) {
+    if (c.tile != q.tile) continue;
+    const double zl = (double)q.zlen, bytes = (double)NX * NY * NZ * 38 * (double)storage_bytes(st);
+    const double us = c.row * (double)(std::min<int64_t>(q.by, NY) + 2);
+    auto wave = [&](int64_t co) {
+      return c.start + (zl + c.planes) * std::max<double>(c.floor, c.base + us * (double)co);
+    };
+    const int64_t m = (q.items + nsm - 1) / nsm;  // CTAs of the busiest SM
+    const double t = (double)(m / per_sm) * wave(per_sm) + (m % per_sm ? wave(m % per_sm) : 0.0);
+    const double mem = bytes < 100e6 ? 0.0 : bytes * (1.0 + 0.35 / zl) / 6.7e6;
+    const double far = bytes < 100e6 ? 1.0 : 1.0 + 0.02 * std::max(0.0, zl / 64 - 1.0);
+    return (std::max(t, mem) + 0.05 * t) * far;
+  }
+  return -1.0;
+}
+
 template <size_t N>
 cudaError_t pick_plan(const TileCost (&cand)[N], int lat, int st, int64_t NX, int64_t NY,
                       int64_t NZ, bool rows, FusedPlan *p) {
@@ -144,7 +199,18 @@ cudaError_t pick_plan(const TileCost (&cand)[N], int lat, int st, int64_t NX, in
       }
     }
   }
-  return found ? cudaSuccess : cudaErrorInvalidValue;
+  if (!found) return cudaErrorInvalidValue;
+  FusedPlan q;
+  if (lat == D3Q19 && st != ST_F64 && !rows && (NX <= 48 || NY < 8 || (st == ST_F32 && NZ <= 8)) &&
+      fused_make_plan(lat, st, 1, NX, NY, NZ, 0, &q) == cudaSuccess) {
+    auto us = [&](const FusedPlan &r) {
+      return st == ST_F32 ? row_us(ROW_F32, r, st, NX, NY, NZ, nsm)
+             : st == ST_F16R || st == ST_BF16R ? row_us(ROW_H16R, r, st, NX, NY, NZ, nsm)
+                                               : row_us(ROW_H16, r, st, NX, NY, NZ, nsm);
+    };
+    if (us(q) >= 0.0 && us(q) < us(*p)) *p = q;
+  }
+  return cudaSuccess;
 }
 }  // namespace
 
