@@ -54,16 +54,16 @@ FALLBACK_HBM_GBS = 6800.0
 # tile scaled by the cells per launch (x8): at 256^3 the lattice is already
 # five times the L2 and the capture's traffic equals the algorithmic bytes.
 NCU_TRAFFIC_PER_LAUNCH = {("d3q19_foam_128", "f32", 25): 277.73e6,
-                          ("d3q19_foam_128", "f64", 6): 622.27e6,
+                          ("d3q19_foam_128", "f64", 6): 621.80e6,
                           ("d3q19_foam_512", "f32", 16): 8 * 2534.55e6,
                           ("d3q19_foam_512", "f16", 24): 8 * 1264.90e6}
 # FP64 storage: the step kernel is bound by the FP64 pipe, not by HBM.  FP64
 # operations per lattice update of its D3Q19 kernel, DADD + DMUL + 2 DFMA as
-# ncu counts them on the 128^3 case (90 + 14 + 2 x 65).  The peak is
+# ncu counts them on the 128^3 case (92.5 + 13.9 + 2 x 67.3).  The peak is
 # measured in the run by lbm_fp64_rate (a DFMA-chain kernel timed with CUDA
 # events); the unit counts give 2 DFMA per SM and cycle x 152 SMs x 2 FLOP x
 # 2.07 GHz = 1.26 TFLOP/s, used only if that measurement fails.
-FP64_FLOP_PER_UPDATE = 234
+FP64_FLOP_PER_UPDATE = 241
 FP64_PEAK_DERIVED_TFLOPS = 2 * 152 * 2 * 2.07e9 / 1e12
 STORAGE_NAME = {"f32": "FP32", "f64": "FP64", "f16": "FP16-offset", "bf16": "BF16-offset"}
 # D3Q19 tile ids of the x-pair kernel (fused_step_kernel_x2)

@@ -81,7 +81,10 @@ typedef enum {
 typedef enum {
   LBM_KERNEL_AUTO = 0,    /* fused kernel with the tuned tile */
   LBM_KERNEL_FUSED = 1,   /* one pass: TMA-staged tiles, psi halo in smem */
-  LBM_KERNEL_TWO_PASS = 2 /* psi field pass + collide/stream pass (AUTO: in one launch, same bits) */
+  /* psi field pass + collide/stream pass.  Where AUTO falls back to it (rows
+   * that are no multiple of 16 bytes) the step is one launch: the same bits in
+   * FP32 arithmetic, FP64 equal to rounding; with mass_residual two launches. */
+  LBM_KERNEL_TWO_PASS = 2
 } lbm_kernel;
 
 /* Optional device allocator.  alloc returns device memory of `bytes` usable

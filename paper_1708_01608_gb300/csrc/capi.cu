@@ -240,11 +240,11 @@ lbm_status sync_and_check(lbm_ctx *c) {
 // array has no pages: the copy then faults them in one after the other and
 // runs at the rate one thread clears memory (26 GB/s), not at that of the
 // link (180 GB/s).  Fresh pages, one copy / backed from here first, then
-// copied: 134 MB 5.1 / 2.9 ms, 537 MB 20 / 9.7 (8
-// threads 4.4 and 14; touching the pages in place of the call is ten times
-// slower, each page being mapped twice under the device's eyes).  MADV_POPULATE_WRITE leaves contents alone and fails
-// without a signal; pages in place, unmapped addresses, registered and device
-// memory are left to the copy.
+// copied: 134 MB 5.1 / 2.9 ms, 537 MB 20 / 9.7 (8 threads 4.4 and 14; touching
+// the pages in place of the call is ten times slower, each page being mapped
+// twice under the device's eyes).  MADV_POPULATE_WRITE leaves contents alone and
+// fails without a signal; pages in place, unmapped addresses, registered and
+// device memory are left to the copy.
 void back_pages(void *dst, size_t bytes) {
 #ifndef MADV_POPULATE_WRITE
   constexpr int MADV_POPULATE_WRITE = 23;

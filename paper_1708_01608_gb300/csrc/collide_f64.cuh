@@ -4,9 +4,11 @@
 // so an FP64 step is bound by that pipe long before HBM: at 128^3 the 304
 // bytes of an update take 94 us per step at the copy bandwidth, the 549 FP64
 // instructions of the former velocity-by-velocity form took 2.285 ms.  This
-// form spends 169 (90 DADD, 14 DMUL, 65 DFMA, halo included): 0.734 ms, the
-// pipe 81 % busy (ncu); D2Q9 at 1024^2 went from 0.599 to 0.183 ms.  With w the edge weight (1/36),
-// m = rho u and one value each per axis a
+// form spends 174 (92 DADD, 14 DMUL, 67 DFMA, halo included): 0.781 ms, the
+// pipe 79 % busy (ncu); D2Q9 at 1024^2 went from 0.599 to 0.201 ms.  (Without
+// the mass terms of relax_pairs and the table's error in psi_f64, 169, 0.752 and
+// 0.184 ms, but twice the former error.)  With w the edge weight (1/36), m = rho u
+// and one value each per axis a
 //   B_a = 3 omega w m_a,  v_a = 1.5 u_a,  Q_a = B_a v_a,
 //   K = omega w rho - (Q_x + Q_y + Q_z)/3,
 // omega f_eq of the rest, an axis and an edge velocity is
@@ -64,9 +66,8 @@ static __device__ const double2 EXP2_64TH[64] = {
 // psi(rho) = rho0 (1 - exp(-rho/rho0)) with the table-driven exponential of
 // Tang (ACM TOMS 15, 1989): x = n ln2/64 + r with |r| <= ln2/128, e^x =
 // 2^(n/64) (1 + r + r^2/2 + ... + r^5/120), the tail below 4e-17.  13 FP64
-// instructions against about 20 with exp() (128^3: 0.786 to 0.743 ms, the
-// density in two chains included).  One of them adds the table entry's own
-// error to r, which gives psi back the error that it has with exp(): of rho0,
+// instructions against about 20 with exp().  One of them adds the table entry's
+// own error to r, which gives psi back the error that it has with exp(): of rho0,
 // in units of 2^-53, rms and largest 0.31 and 0.89 (rho0 = 1; exp() 0.32 and
 // 0.90, without e 0.34 and 1.24) and 0.38 and 1.27 (others; exp() 0.49 and
 // 1.66).  The range test is on integers; outside it (and for NaN) exp()

@@ -128,16 +128,16 @@ __global__ void __launch_bounds__(TPB) k_ml_psi(const MlArgs<T> a, T *psi) {
 // collide_f64.cuh.  Us per step with three lattices, a launch of one thread
 // per cell for psi and one for the collision of all lattices (844 FP64
 // instructions per cell, 43 CTAs at 104^2) against this form: FP64 104^2 96.9
-// / 11.8, 500^2 698 / 208, D3Q19 64x64x48 912 / 239; FP32 104^2 16.4 / 3.7,
-// 1000^2 161 / 118, 64x64x48 66.6 / 27.2.
+// / 12.3, 500^2 698 / 218, D3Q19 64x64x48 912 / 244; FP32 104^2 16.4 / 3.4,
+// 1000^2 161 / 113, 64x64x48 66.6 / 27.1.
 //
 // Forms: psi of the tile and a one-cell halo formed in shared memory, one launch
 // per step (ML_TILE, D2Q9); psi from k_ml_psi, the CTA's cells of one row
 // (ML_ROW) or in memory order (ML_RUN; D3Q19).
 enum { ML_TILE = 0, ML_ROW = 1, ML_RUN = 2 };
 template <int LAT, class T, int FORM>
-__global__ void __launch_bounds__(ML_TPB, sizeof(T) == 8 ? 2 : 3) k_ml_step(const MlArgs<T> a, const MlTile tl,
-                                                 const T *psi_field) {
+__global__ void __launch_bounds__(ML_TPB, sizeof(T) == 8 ? 2 : 3)
+    k_ml_step(const MlArgs<T> a, const MlTile tl, const T *psi_field) {
   using L = Lattice<LAT>;
   constexpr int Q = L::Q;
   constexpr bool FIELD = FORM != ML_TILE;

@@ -25,8 +25,8 @@
 // collision of collide_f64.cuh.
 //
 // us per step, two-pass / this: 201x150x99 FP32 168 / 121, FP16 164 / 97;
-// 33x35x31 FP32 10.3 / 4.9; 93^3 FP64 772 / 451; D2Q9 201^2 FP32 10.3 / 3.0,
-// 1401x1203 68 / 25, 129^2 FP64 27 / 11; the allocation-free step at
+// 33x35x31 FP32 10.3 / 4.9; 93^3 FP64 772 / 461; D2Q9 201^2 FP32 10.3 / 3.0,
+// 1401x1203 68 / 25, 129^2 FP64 27 / 11.5; the allocation-free step at
 // 127x101x90 54 / 43.5.  Blocks of 32 x 8 threads, three per SM, against 32 x
 // 12, two per SM (124 and 105 at 201x150x99) and 32 x 24 (144 and 118);
 // without the plane in flight 129 and 112.

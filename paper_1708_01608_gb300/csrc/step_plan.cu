@@ -77,14 +77,14 @@ constexpr TileCost COST_H16[] = {{24, 1.0f, 1.75f, 1.2f, 1.95f}, {23, 1.0f, 1.75
 // 16-bit with the rounding residual: 256^3 460 / 283
 constexpr TileCost COST_H16R[] = {{23, 1.2f, 2.1f, 1.7f, 2.4f}, {24, 1.2f, 2.1f, 1.7f, 2.4f},
                                   {2, 0.55f, 4.5f, 1.7f, 4.5f}};
-// FP64 is bound by the FP64 pipe, which the CTAs of an SM share: 32^3 64 / 22
+// FP64 is bound by the FP64 pipe, which the CTAs of an SM share: 32^3 64 / 24
 constexpr TileCost COST_F64[] = {{6, 0.0f, 49.0f, 0.0f, 49.0f}, {7, 0.0f, 49.0f, 0.0f, 49.0f},
                                  {2, 0.0f, 54.0f, 0.0f, 54.0f}};
 // D2Q9, FP32 and 16-bit (the floor adds here: co-resident rows overlap):
 // 64^2 4.6 / 2.7, 200^2 4.9 / 3.2, 512^2 7.4 / 5.6, 2000^2 56.5 / 50.5
 constexpr TileCost COST_2D[] = {{4, 0.35f, 0.5f, 0.35f, 0.5f}, {6, 0.35f, 0.6f, 0.35f, 0.6f},
                                 {3, 0.33f, 0.8f, 0.33f, 0.8f}};
-// D2Q9 FP64: 64^2 21.1 / 8.8, 128^2 22.0 / 9.2, 512^2 60 / 54
+// D2Q9 FP64: 64^2 21.1 / 9.2, 128^2 22.0 / 9.7, 512^2 60 / 56.5
 constexpr TileCost COST_2D_F64[] = {{1, 2.6f, 25.5f, 2.6f, 25.5f}, {3, 2.6f, 25.5f, 2.6f, 25.5f}};
 
 // Narrow lattices with D3Q19 and FP32 arithmetic: rows of 4 to 48 cells, fewer
