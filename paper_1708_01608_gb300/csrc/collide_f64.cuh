@@ -7,7 +7,7 @@
 // form spends 174 (92 DADD, 14 DMUL, 67 DFMA, halo included): 0.781 ms, the
 // pipe 79 % busy (ncu); D2Q9 at 1024^2 went from 0.599 to 0.201 ms.  (Without
 // the mass terms of relax_pairs and the table's error in psi_f64, 169, 0.752 and
-// 0.184 ms, but twice the former error.)  With w the edge weight (1/36), m = rho u
+// 0.189 ms, but twice the former error.)  With w the edge weight (1/36), m = rho u
 // and one value each per axis a
 //   B_a = 3 omega w m_a,  v_a = 1.5 u_a,  Q_a = B_a v_a,
 //   K = omega w rho - (Q_x + Q_y + Q_z)/3,
@@ -93,7 +93,7 @@ __device__ __forceinline__ bool rcp_overflows(double b) {
   return (__double2hiint(b) & 0x7fffffff) < 0x00100000;
 }
 __device__ __forceinline__ bool rcp_overflows(float b) {
-  return (__float_as_int(b) & 0x7fffffff) < 0x00800000;
+  return fabsf(b) < 0x1p-126f;
 }
 
 // Density of one cell from its Q values, in two chains (half the latency of

@@ -564,7 +564,7 @@ __device__ __forceinline__ MarchArgs march_args_of(const FusedMaps &tm, const St
 // item = zc * tiles + tt, so the CTAs resident together cover neighbouring
 // columns at the same planes (their halo rows meet in L2).
 // 256-thread tiles are register-limited to 3 CTAs per SM (FP64: shared
-// memory holds 2, which leaves 128 registers), the larger ones run one
+// memory holds 2 at most, which leaves 128 registers), the larger ones run one
 template <int LAT, int ST, int BX, int BY, int NS>
 __global__ void __launch_bounds__(BX *BY, BX *BY <= 256 ? (ST == ST_F64 ? 2 : 3) : 1)
     fused_step_kernel(const __grid_constant__ FusedMaps tm, const StepArgs a, const int tiles_x,
